@@ -202,6 +202,16 @@ __device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v) {
   asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v) : "memory");
 }
 
+// The state after decoding the symbol of table entry e (sym | bias << 8 |
+// (freq - 1) << 20): freq * (x >> 12) + bias. With q = freq - 1 and e >> 8 =
+// q << 12 | bias this is q * ((x >> 12) - 4096) + (x >> 12) + (e >> 8): no
+// mask for the bias and no increment of q, one instruction less per step of
+// an issue-bound loop (1 GiB FASTQ 1.511 -> 1.495 ms).
+__device__ __forceinline__ uint32_t rans_next(uint32_t x, uint32_t e) {
+  const uint32_t xh = x >> kScaleBits;
+  return (e >> 20) * (xh - kScale) + (xh + (e >> 8));
+}
+
 // The command staging area of a warp: shared memory (kShared, read and
 // written through its shared-window address), or a generic pointer to shared
 // memory or to the warp's global slot for segments whose command streams do
@@ -386,7 +396,7 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
     if (active) {
       const uint32_t e = entry((cls << kScaleBits) | (x & (kScale - 1)));
       sym = e & 0xFFu;
-      x = ((e >> 20) + 1u) * (x >> kScaleBits) + ((e >> 8) & 0xFFFu);
+      x = rans_next(x, e);
     }
     renorm(active && x < kRansL);
     return sym;
@@ -415,7 +425,7 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
     // four steps inside one class: the table row is known for all lanes
     auto cls_step = [&](uint32_t row) -> uint32_t {
       const uint32_t e = entry(row | (x & (kScale - 1)));
-      x = ((e >> 20) + 1u) * (x >> kScaleBits) + ((e >> 8) & 0xFFFu);
+      x = rans_next(x, e);
       renorm(x < kRansL);
       return e & 0xFFu;
     };
@@ -502,7 +512,7 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
     };
     auto lit_rans = [&]() -> uint32_t {
       const uint32_t e = entry((3u << kScaleBits) | (x & (kScale - 1)));
-      x = ((e >> 20) + 1u) * (x >> kScaleBits) + ((e >> 8) & 0xFFFu);
+      x = rans_next(x, e);
       renorm(x < kRansL);
       return e;
     };
@@ -554,7 +564,7 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
       uint32_t e = 0;
       if (active) {
         e = entry((3u << kScaleBits) | (x & (kScale - 1)));
-        x = ((e >> 20) + 1u) * (x >> kScaleBits) + ((e >> 8) & 0xFFFu);
+        x = rans_next(x, e);
       }
       renorm(active && x < kRansL);
       if (active) outK[o] = (uint8_t)e;
