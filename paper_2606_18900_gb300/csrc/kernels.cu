@@ -49,6 +49,24 @@ __device__ __forceinline__ void st_release(uint64_t *p, uint64_t v) {
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// the same within the CTA, on a word in shared memory
+__device__ __forceinline__ uint32_t ld_acquire_cta(const uint32_t *p) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_acquire_cta8(const uint8_t *p) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared.u8 %0, [%1];" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release_cta8(uint8_t *p, uint32_t v) {
+  asm volatile("st.release.cta.shared.u8 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_release_cta(uint32_t *p, uint32_t v) {
+  asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+}
+
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t *p) {
   uint32_t v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -175,6 +193,50 @@ __device__ __forceinline__ void realign16(uint4 X, uint4 Y, uint32_t c, uint32_t
   for (int j = 0; j < 4; ++j) r[j] = __funnelshift_r(s1[j], s1[j + 1], sh);
 }
 
+// Bytes [o, o + n) of the 16-byte block at `to` (16-byte aligned), n < 16, from
+// the block r.
+__device__ __forceinline__ void store_piece(uint8_t *to, const uint32_t r[4], uint32_t o, uint32_t n) {
+  // bytes [o, o + n) of the block as naturally aligned pieces of
+  // 1, 2, 4 and 8 bytes (a scattered store costs the memory
+  // pipeline one pass per line it touches, whatever its width)
+  auto wd = [&](uint32_t i) { return i & 2 ? (i & 1 ? r[3] : r[2]) : (i & 1 ? r[1] : r[0]); };
+  if (o == 0 || o + n == 16) {
+    // the first or last block of a match: one end of the bytes is
+    // an end of the block, and the pieces are the set bits of n,
+    // rising in size from o when the bytes end at the block's end,
+    // falling from 0 when they start at its start (four store
+    // instructions per warp)
+    const bool rise = o != 0;
+    if (n & 8) *reinterpret_cast<uint2 *>(to + (rise ? 8 : 0)) = rise ? make_uint2(r[2], r[3]) : make_uint2(r[0], r[1]);
+    if (n & 4) {
+      const uint32_t a = rise ? o + (n & 3) : (n & 8);
+      *reinterpret_cast<uint32_t *>(to + a) = wd(a >> 2);
+    }
+    if (n & 2) {
+      const uint32_t a = rise ? o + (n & 1) : (n & 12);
+      *reinterpret_cast<uint16_t *>(to + a) = (uint16_t)(wd(a >> 2) >> (8 * (a & 2)));
+    }
+    if (n & 1) {
+      const uint32_t a = rise ? o : (n & 14);
+      to[a] = (uint8_t)(wd(a >> 2) >> (8 * (a & 3)));
+    }
+  } else {
+    // both ends inside the block (a match shorter than 16 bytes):
+    // rising in size up to the first boundary that the next piece
+    // would cross, then falling (eight store instructions)
+    uint32_t a = o;
+    const uint32_t e = o + n;
+    if ((a & 1) && a < e) { to[a] = (uint8_t)(wd(a >> 2) >> (8 * (a & 3))); a += 1; }
+    if ((a & 2) && a + 2 <= e) { *reinterpret_cast<uint16_t *>(to + a) = (uint16_t)(wd(a >> 2) >> (8 * (a & 2))); a += 2; }
+    if ((a & 4) && a + 4 <= e) { *reinterpret_cast<uint32_t *>(to + a) = wd(a >> 2); a += 4; }
+    if ((a & 8) && a + 8 <= e) { *reinterpret_cast<uint2 *>(to + a) = make_uint2(r[2], r[3]); a += 8; }
+    if (a + 8 <= e) { *reinterpret_cast<uint2 *>(to + a) = (a & 8) ? make_uint2(r[2], r[3]) : make_uint2(r[0], r[1]); a += 8; }
+    if (a + 4 <= e) { *reinterpret_cast<uint32_t *>(to + a) = wd(a >> 2); a += 4; }
+    if (a + 2 <= e) { *reinterpret_cast<uint16_t *>(to + a) = (uint16_t)(wd(a >> 2) >> (8 * (a & 2))); a += 2; }
+    if (a < e) to[a] = (uint8_t)(wd(a >> 2) >> (8 * (a & 3)));
+  }
+}
+
 // Per-warp shared table of the matches copied in one round.
 struct MatchTable {
   uint64_t src[32];
@@ -194,6 +256,16 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds_u8(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint4 lds_v4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
   return v;
 }
 __device__ __forceinline__ void sts_u8(uint32_t a, uint32_t v) {
@@ -306,12 +378,19 @@ __device__ unsigned long long g_phase_cycles[16];
 // segments' flags, then match copies in rounds: a round copies every pending
 // match whose source does not overlap the output of an earlier pending match,
 // the bytes of the round spread over all lanes; (5) publish.
-template <bool kSmemLut, int kMode, bool kSharedStage>
-__device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const DevArchive &A, const OutView &V,
-                                                    uint32_t seg, uint32_t epoch, const uint32_t *lut,
-                                                    uint32_t lut_s, const Stage<kSharedStage> st, MatchTable *mt,
-                                                    uint32_t ring_s, int lane, const SegRec &d, uint64_t *ph,
-                                                    uint64_t &ph_t) {
+//
+// entropy_phases is (1) to (3): false when the segment is corrupt (or its
+// page absent); the command records are then in the stage.
+// kStaged: the literals are only decoded, literal k to byte tot_m + k of the
+// segment's copy in shared memory at out_s (tot_m: the segment's match bytes;
+// place_literals moves them from there), and *progress counts the literals
+// decoded so far. after_parse(ok, tot_m) is called between (2) and (3).
+template <bool kSmemLut, int kMode, bool kSharedStage, bool kStaged, class AfterParse>
+__device__ __forceinline__ bool entropy_phases(const DevArchive &A, const OutView &V, uint32_t seg,
+                                               const uint32_t *lut, uint32_t lut_s, const Stage<kSharedStage> st,
+                                               uint32_t ring_s, uint32_t out_s, uint32_t *progress,
+                                               AfterParse after_parse, int lane, const SegRec &d, uint64_t *ph,
+                                               uint64_t &ph_t) {
   (void)ph;
   (void)ph_t;
   const uint32_t log2_S = A.log2_S;
@@ -323,12 +402,6 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
   // the segment's own output is contiguous in every view
   uint8_t *const out = at(V, seg_start, log2_S);
   bool ok = out != nullptr;
-  // aligned 16-byte blocks of the view never straddle a segment (hence no ring
-  // wrap or page boundary either)
-  const bool vec =
-      log2_S >= 4 && (kMode == kViewPaged  ? (reinterpret_cast<uintptr_t>(V.slot_base) & 15) == 0
-                      : kMode == kViewRing ? ((reinterpret_cast<uintptr_t>(V.base) | V.origin) & 15) == 0
-                                           : ((reinterpret_cast<uintptr_t>(V.base) - V.origin) & 15) == 0);
 
   // ---------------------------------------------------------------- rANS
   const uint8_t *pl = A.payload + d.payload_off;
@@ -489,12 +562,60 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
   __syncwarp();
   PHASE_MARK(1);
 
+  after_parse(ok, tot_m);
+
   // (3) literals. K0: literal number of lane 0 in the current step; E: end of
   // the literal run of command cu (literal number), the next boundary; Sc:
   // match bytes before the literals from the current boundary on (the
   // cumulative match length through command cu - 1); outK: the output
   // address of literal K0 before any match byte.
-  if (ok) {
+  if (kStaged && ok) {
+    uint32_t to = out_s + tot_m + (uint32_t)lane;  // where the lane's next literal goes
+    uint32_t n_done = 0;
+    auto step = [&](bool active) -> uint32_t {
+      // the words from wr on, one per lane: read before the chain needs them,
+      // and handed out by a shuffle, which is shorter than an indexed read
+      const uint32_t words = lds_u16(wr + 2 * lane);
+      uint32_t e = 0;
+      if (active) {
+        e = entry((3u << kScaleBits) | (x & (kScale - 1)));
+        x = rans_next(x, e);
+      }
+      const bool need = active && x < kRansL;
+      const uint32_t m = __ballot_sync(kFull, need);
+      const uint32_t w = __shfl_sync(kFull, words, __popc(m & lt));
+      if (need) x = __byte_perm(w, x, 0x5410);  // x << 16 | w
+      wr += 2 * __popc(m);
+      return e;
+    };
+    auto tell = [&]() {
+      __syncwarp();
+      if (lane == 0) st_release_cta(progress, n_done);
+    };
+    if (b3 & 31u) {  // the crossing step, decoded in (1): its literals are lanes b3 mod 32 on
+      const uint32_t l0 = b3 & 31u;
+      if ((uint32_t)lane >= l0 && t0 - 32 + lane < n_sym) sts_u8(to - l0, pend);
+      n_done = min(32 - l0, nl);
+      to += 32 - l0;
+    }
+    for (; t0 + 128 <= n_sym; t0 += 128) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sts_u8(to + 32 * u, step(true));
+      to += 128;
+      n_done += 128;
+      advance();
+      tell();
+    }
+    for (; t0 < n_sym; t0 += 32) {
+      const bool active = t0 + lane < n_sym;
+      const uint32_t e = step(active);
+      if (active) sts_u8(to, e);
+      to += 32;
+      advance();
+    }
+    n_done = nl;
+    tell();
+  } else if (ok) {
     int K0 = (b3 & 31u) ? (int)(b3 & ~31u) - (int)b3 : 0;
     uint32_t cu = 0, rec = st.u32(0), Sc = 0;
     int E = (int)(rec & 0xFFFFu);
@@ -578,12 +699,112 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
   if (!__all_sync(kFull, x == kRansL) || wb != 2 * nw) ok = false;
   __syncwarp();
   PHASE_MARK(2);
+  return ok;
+}
 
-  // (4) matches
-  const uint32_t my_level = d.level;
+// Named barriers of a team. The forms without .aligned: the code before them
+// branches by lane, and a warp that reached an aligned barrier in two parts
+// would be counted twice.
+__device__ __forceinline__ void named_sync(uint32_t id, uint32_t threads) {
+  __syncwarp();
+  asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_arrive(uint32_t id, uint32_t threads) {
+  __syncwarp();
+  asm volatile("barrier.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// A team of warps that share one segment (staged_kernel): in the shared
+// memory of the CTA.
+constexpr uint32_t kTeamBytes = 416;  // a segment has at most 16384 / 5 commands: 410 groups of 8
+struct TeamState {
+  uint32_t seg;                // segment being decoded; kNoSeg ends the team
+  uint32_t fail;               // set by the warp that finds the segment corrupt or a wait too long
+  uint32_t lits;               // literals decoded so far
+  uint32_t tot_m;              // match bytes of the segment
+  uint8_t done[kTeamBytes];    // bit k of byte j: the match of command 8 j + k is in place
+};
+constexpr uint32_t kNoSeg = 0xFFFFFFFFu;
+constexpr uint32_t kMaxTeams = 6;  // teams of a CTA: two named barriers each, of 1 .. 15
+constexpr uint32_t kMaxTeam = 16;  // warps per team
+constexpr uint32_t kStagedThreads = 768;
+constexpr uint32_t kStagedSmem = 228352;  // dynamic shared memory of staged_kernel; its static part is below 4 KiB
+
+__device__ __forceinline__ uint32_t ld_vol(const uint32_t *p) { return *const_cast<const volatile uint32_t *>(p); }
+
+// The literals of a segment that a team's first warp is decoding, moved from
+// byte tot_m + k of the copy at out_s to their places, 128 at a time behind
+// the decoder. A literal's place is never after where it was decoded to, and
+// never after an earlier literal's source, so moving the blocks in order (each
+// read before it is written) keeps what is still to be moved. False when the
+// decoder gave up.
+__device__ __forceinline__ bool place_literals(const Stage<true> st, const TeamState *ts, uint32_t out_s, uint32_t nl,
+                                               uint64_t deadline, uint32_t *err, int lane) {
+  const uint32_t tot_m = ts->tot_m, from = out_s + tot_m + (uint32_t)lane;
+  // rec: the next run end (literal number, match bytes through its command);
+  // ahead: the record after it, read early (the stage is readable past the
+  // sentinel, and what follows it is never used)
+  uint32_t cu = 0, rec = st.u32(0), ahead = st.u32(4), S = 0;
+  for (uint32_t K = 0; K < nl && S != tot_m; K += 128) {
+    const uint32_t want = min(K + 128, nl);
+    for (uint32_t spin = 0; ; ++spin) {
+      if (__all_sync(kFull, ld_acquire_cta(&ts->lits) >= want)) break;
+      uint32_t why = 0;
+      if (lane == 0 && (spin & 63) == 63) why = ld_vol(&ts->fail) ? 1u : now_ns() > deadline ? 2u : 0u;
+      why = __shfl_sync(kFull, why, 0);
+      if (why) {
+        if (why == 2 && lane == 0) latch(err, kErrTimeout);
+        return false;
+      }
+      __nanosleep(40);
+    }
+    uint32_t v[4], o[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[u] = K + 32 * u + lane < nl ? lds_u8(from + K + 32 * u) : 0u;
+      o[u] = S;
+    }
+    __syncwarp();
+    while ((rec & 0xFFFFu) < K + 128) {  // a run end inside the block (the sentinel's lies beyond every literal)
+      const int D = (int)((rec & 0xFFFFu) - K);
+      S = rec >> 16;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (lane + 32 * u >= D) o[u] = S;
+      ++cu;
+      rec = ahead;
+      ahead = st.u32(4 * cu + 4);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (K + 32 * u + lane < nl) sts_u8(out_s + K + 32 * u + lane + o[u], v[u]);
+    __syncwarp();
+  }
+  return true;
+}
+
+// Phase (4) of a segment whose entropy phases are done, by one warp, in the
+// view. False when a command is corrupt or a wait gave up.
+template <int kMode, bool kSharedStage>
+__device__ __forceinline__ bool match_phase(const DecodeLaunch &L, const DevArchive &A, const OutView &V, uint32_t seg,
+                                            uint32_t epoch, const Stage<kSharedStage> st, MatchTable *mt, int lane,
+                                            uint32_t nc, uint32_t my_level, uint64_t *ph, uint64_t &ph_t) {
+  (void)ph;
+  (void)ph_t;
+  const uint32_t log2_S = A.log2_S, W = A.W;
+  const uint64_t seg_start = (uint64_t)seg << log2_S;
+  const uint32_t offs = 4 * nc + 4;
+  uint8_t *const out = at(V, seg_start, log2_S);
+  bool ok = true;
+  // aligned 16-byte blocks of the view never straddle a segment (hence no ring
+  // wrap or page boundary either)
+  const bool vec =
+      log2_S >= 4 && (kMode == kViewPaged  ? (reinterpret_cast<uintptr_t>(V.slot_base) & 15) == 0
+                      : kMode == kViewRing ? ((reinterpret_cast<uintptr_t>(V.base) | V.origin) & 15) == 0
+                                           : ((reinterpret_cast<uintptr_t>(V.base) - V.origin) & 15) == 0);
   const uint64_t deadline = now_ns() + L.wait_ns;
   uint32_t mbase = 0;  // match bytes before the chunk
-  for (uint32_t c0 = 0; ok && c0 < nc; c0 += 32) {
+  for (uint32_t c0 = 0; c0 < nc; c0 += 32) {
     const uint32_t c = c0 + lane;
     const bool valid = c < nc;
     uint32_t ml = 0, lend = 0, cum = 0;
@@ -746,45 +967,7 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
           if (n == 16) {
             *reinterpret_cast<uint4 *>(to) = make_uint4(r[0], r[1], r[2], r[3]);
           } else {
-            // bytes [o, o + n) of the block as naturally aligned pieces of
-            // 1, 2, 4 and 8 bytes (a scattered store costs the memory
-            // pipeline one pass per line it touches, whatever its width)
-            auto wd = [&](uint32_t i) { return i & 2 ? (i & 1 ? r[3] : r[2]) : (i & 1 ? r[1] : r[0]); };
-            if (o == 0 || o + n == 16) {
-              // the first or last block of a match: one end of the bytes is
-              // an end of the block, and the pieces are the set bits of n,
-              // rising in size from o when the bytes end at the block's end,
-              // falling from 0 when they start at its start (four store
-              // instructions per warp)
-              const bool rise = o != 0;
-              if (n & 8) *reinterpret_cast<uint2 *>(to + (rise ? 8 : 0)) = rise ? make_uint2(r[2], r[3]) : make_uint2(r[0], r[1]);
-              if (n & 4) {
-                const uint32_t a = rise ? o + (n & 3) : (n & 8);
-                *reinterpret_cast<uint32_t *>(to + a) = wd(a >> 2);
-              }
-              if (n & 2) {
-                const uint32_t a = rise ? o + (n & 1) : (n & 12);
-                *reinterpret_cast<uint16_t *>(to + a) = (uint16_t)(wd(a >> 2) >> (8 * (a & 2)));
-              }
-              if (n & 1) {
-                const uint32_t a = rise ? o : (n & 14);
-                to[a] = (uint8_t)(wd(a >> 2) >> (8 * (a & 3)));
-              }
-            } else {
-              // both ends inside the block (a match shorter than 16 bytes):
-              // rising in size up to the first boundary that the next piece
-              // would cross, then falling (eight store instructions)
-              uint32_t a = o;
-              const uint32_t e = o + n;
-              if ((a & 1) && a < e) { to[a] = (uint8_t)(wd(a >> 2) >> (8 * (a & 3))); a += 1; }
-              if ((a & 2) && a + 2 <= e) { *reinterpret_cast<uint16_t *>(to + a) = (uint16_t)(wd(a >> 2) >> (8 * (a & 2))); a += 2; }
-              if ((a & 4) && a + 4 <= e) { *reinterpret_cast<uint32_t *>(to + a) = wd(a >> 2); a += 4; }
-              if ((a & 8) && a + 8 <= e) { *reinterpret_cast<uint2 *>(to + a) = make_uint2(r[2], r[3]); a += 8; }
-              if (a + 8 <= e) { *reinterpret_cast<uint2 *>(to + a) = (a & 8) ? make_uint2(r[2], r[3]) : make_uint2(r[0], r[1]); a += 8; }
-              if (a + 4 <= e) { *reinterpret_cast<uint32_t *>(to + a) = wd(a >> 2); a += 4; }
-              if (a + 2 <= e) { *reinterpret_cast<uint16_t *>(to + a) = (uint16_t)(wd(a >> 2) >> (8 * (a & 2))); a += 2; }
-              if (a < e) to[a] = (uint8_t)(wd(a >> 2) >> (8 * (a & 3)));
-            }
+            store_piece(to, r, o, n);
           }
         } else {
           const uint32_t o = (uu - mt->start[m]) << 4;
@@ -810,14 +993,198 @@ __device__ __forceinline__ void decode_segment_impl(const DecodeLaunch &L, const
     }
     PHASE_MARK(4);
   }
-  if (!ok && lane == 0 && ld_relaxed(L.err) == 0) latch(L.err, kErrCorrupt);
+  return ok;
+}
 
-  PHASE_COUNT(9, 1);
-  // ------------------------------------------------------------- publish
-  // (no fence per lane: the warp barrier orders every lane's stores before
-  // lane 0's release store, and release is cumulative)
-  __syncwarp();
-  if (lane == 0 && ok && !(A.blocked && A.blocked[seg])) st_release(A.flags + seg, (uint64_t)d.level << 32 | epoch);
+// A match being copied by a team: ml bytes from absolute position src to
+// offset doff of the segment's copy.
+struct TeamMatch {
+  uint64_t src;
+  uint32_t doff, ml;
+  // the copy's aligned 16-byte blocks that it touches
+  __device__ __forceinline__ uint32_t blocks() const { return ((doff & 15u) + ml + 15) >> 4; }
+};
+
+// Blocks k0, k0 + step, ... of match m, into the segment's copy at out_s. What
+// lies in this segment is read from the copy, the rest from the view. vec: the
+// view's 16-byte blocks are aligned in memory, and a block is built from the
+// one or two aligned blocks (each in one segment) that hold its bytes; else
+// the bytes are copied one by one.
+template <int kMode>
+__device__ __forceinline__ void copy_blocks(const DevArchive &A, const OutView &V, uint64_t seg_start, uint32_t out_s,
+                                            const TeamMatch &m, uint32_t k0, uint32_t step, bool vec) {
+  if (!vec) {
+#pragma unroll 1
+    for (uint32_t j = k0; j < m.ml; j += step)
+      sts_u8(out_s + m.doff + j, m.src + j >= seg_start ? lds_u8(out_s + (uint32_t)(m.src + j - seg_start))
+                                                       : (uint32_t)*src_at<kMode>(V, m.src + j, A.log2_S));
+    return;
+  }
+  auto block = [&](uint64_t q) -> uint4 {
+    if (q >= seg_start) return lds_v4(out_s + (uint32_t)(q - seg_start));
+    const uint8_t *p = src_at<kMode>(V, q, A.log2_S);
+    return kMode != kViewPaged || p ? *reinterpret_cast<const uint4 *>(p) : make_uint4(0, 0, 0, 0);
+  };
+  for (uint32_t k = k0; k < m.blocks(); k += step) {
+    const uint32_t b16 = (m.doff & ~15u) + 16 * k;
+    const uint32_t a0 = max(m.doff, b16), a1 = min(m.doff + m.ml, b16 + 16), o = a0 - b16, n = a1 - a0;
+    const uint64_t P = m.src + (a0 - m.doff);
+    const uint32_t dl = (uint32_t)P & 15u;
+    uint4 X = make_uint4(0, 0, 0, 0), Y = X;
+    const uint64_t q = P - dl;
+    if (dl >= o) {
+      X = block(q);
+      if (dl + n > 16) Y = block(q + 16);
+    } else {
+      Y = block(q);
+    }
+    uint32_t r[4];
+    realign16(X, Y, (dl - o) & 15u, r);
+    uint8_t *to = reinterpret_cast<uint8_t *>(__cvta_shared_to_generic(out_s + b16));
+    if (n == 16) *reinterpret_cast<uint4 *>(to) = make_uint4(r[0], r[1], r[2], r[3]);
+    else store_piece(to, r, o, n);
+  }
+}
+
+// Phase (4) by a team of T warps, in the segment's copy in shared memory at
+// out_s. Commands go to the warps in batches of B (batch j to warp j mod T,
+// each warp's in order), one to a lane; B is 8, 16 or 32, the least that takes
+// all commands in one batch per warp. A match is copied, by four lanes, as soon as
+// its source segments are published and the earlier matches of this segment
+// that it reads are in place (ts->done): it waits for nothing else, so the
+// length of this phase is the longest chain of such matches and not their
+// number, and since every wait is for a lower command or a lower level, the
+// waits end. Matches of more than 16 blocks are copied by the whole warp.
+// False when a command is corrupt or a wait gave up.
+template <int kMode>
+__device__ __forceinline__ bool match_phase_team(const DecodeLaunch &L, const DevArchive &A, const OutView &V,
+                                                 uint32_t seg, uint32_t epoch, const Stage<true> st, int lane,
+                                                 uint32_t nc, uint32_t my_level, TeamState *ts, uint32_t out_s,
+                                                 uint32_t first, uint32_t T) {
+  const uint32_t log2_S = A.log2_S, W = A.W, offs = 4 * nc + 4;
+  const uint64_t seg_start = (uint64_t)seg << log2_S;
+  const bool vec =
+      log2_S >= 4 && (kMode == kViewPaged  ? (reinterpret_cast<uintptr_t>(V.slot_base) & 15) == 0
+                      : kMode == kViewRing ? ((reinterpret_cast<uintptr_t>(V.base) | V.origin) & 15) == 0
+                                           : ((reinterpret_cast<uintptr_t>(V.base) - V.origin) & 15) == 0);
+  const uint64_t deadline = now_ns() + L.wait_ns;
+  const uint32_t B = 8 * T >= nc ? 8u : 16 * T >= nc ? 16u : 32u;
+  for (uint32_t c0 = B * first; c0 < nc; c0 += B * T) {
+    const uint32_t c = c0 + (uint32_t)lane;
+    bool pending = (uint32_t)lane < B && c < nc, bad = false;
+    uint32_t ml = 0, doff = 0;
+    uint64_t src = 0;
+    // the earlier commands [jlo, jhi] whose matches this one reads
+    uint32_t jlo = 1, jhi = 0;
+    const uint64_t *f0 = nullptr, *f1 = nullptr;  // flags of the source segments
+    if (pending) {
+      const uint32_t rec = st.u32(4 * c), before = c ? st.u32(4 * c - 4) >> 16 : 0u;
+      src = W == 4 ? (uint64_t)st.u32(offs + 4 * c) : st.le(offs + W * c, W);
+      ml = (rec >> 16) - before;
+      doff = (rec & 0xFFFFu) + before;
+      const uint64_t q0 = src >> log2_S, q1 = (src + ml - 1) >> log2_S;
+      // (the parse has checked the command; these bounds keep every access below in place)
+      bad = q1 >= A.n_seg || ml - 1 >= 1u << log2_S || doff + ml > 1u << log2_S;
+      if (!bad && q0 != seg) f0 = A.flags + q0;
+      if (!bad && q1 != q0 && q1 != seg) f1 = A.flags + q1;
+      if (kMode == kViewPaged) bad |= (f0 && V.page[q0] == 0xFFFFFFFFu) || (f1 && V.page[q1] == 0xFFFFFFFFu);
+      if (src + ml > seg_start) {
+        // command j's match ends at offset C(j) = its record's two halves:
+        // jlo is the first with C > src, jhi the first with C >= src + ml,
+        // or the one before if that match starts after the source
+        const uint32_t s_rel = src > seg_start ? (uint32_t)(src - seg_start) : 0u;
+        const uint32_t e_rel = (uint32_t)(src + ml - seg_start);
+        auto end_of = [&](uint32_t j) {
+          const uint32_t r = st.u32(4 * j);
+          return (r & 0xFFFFu) + (r >> 16);
+        };
+        uint32_t a = 0, b = 0;
+        for (uint32_t s = 1u << (31 - __clz(c | 1u)); s; s >>= 1) {
+          if (a + s <= c && end_of(a + s - 1) <= s_rel) a += s;
+          if (b + s <= c && end_of(b + s - 1) < e_rel) b += s;
+        }
+        // (b <= c: this command's own match starts at or after src + ml)
+        if (b == c || (st.u32(4 * b) & 0xFFFFu) + (b ? st.u32(4 * b - 4) >> 16 : 0u) >= e_rel) --b;
+        if ((int)a <= (int)b) jlo = a, jhi = b;
+      }
+    }
+    bool look = true;  // read the flags (an L2 round trip) only when nothing else is left to do
+    for (uint32_t spin = 0;; ++spin) {
+      if (look && pending) {
+        // each flag is read until it has this call's epoch; a source segment
+        // must have a lower level than ours (a wait on any other could not end)
+        const uint64_t v0 = f0 ? ld_acquire(f0) : epoch, v1 = f1 ? ld_acquire(f1) : epoch;
+        if (f0) bad |= (uint32_t)(v0 >> 32) >= my_level;
+        if (f1) bad |= (uint32_t)(v1 >> 32) >= my_level;
+        if ((uint32_t)v0 == epoch) f0 = nullptr;
+        if ((uint32_t)v1 == epoch) f1 = nullptr;
+      }
+      bool ready = pending && !f0 && !f1;
+      if (ready) {
+        while (jlo <= jhi) {  // (in place ones are passed for good)
+          const uint32_t m = ld_acquire_cta8(ts->done + (jlo >> 3));
+          if (!(m >> (jlo & 7u) & 1u)) break;
+          ++jlo;
+        }
+        if (jlo <= jhi) ready = false;
+      }
+      if (__any_sync(kFull, bad)) return false;
+      const uint32_t rm = __ballot_sync(kFull, ready);
+      if (rm) {
+        const uint32_t big = __ballot_sync(kFull, ready && TeamMatch{src, doff, ml}.blocks() > 16);
+        __syncwarp();  // (lanes read behind the acquires of the lanes that hold the matches)
+        auto match_of = [&](int l) {
+          return TeamMatch{__shfl_sync(kFull, src, l), __shfl_sync(kFull, doff, l), __shfl_sync(kFull, ml, l)};
+        };
+#pragma unroll 1
+        for (int g = 0; g < (int)B; g += 8) {
+          const uint32_t some = rm & ~big & (0xFFu << g);
+          if (!some) continue;
+          const int l = g + (lane >> 2);
+          const TeamMatch m = match_of(l);
+          if (some >> l & 1u) copy_blocks<kMode>(A, V, seg_start, out_s, m, (uint32_t)lane & 3u, 4, vec);
+          __syncwarp();
+        }
+#pragma unroll 1
+        for (uint32_t r = big; r; r &= r - 1)
+          copy_blocks<kMode>(A, V, seg_start, out_s, match_of(__ffs((int)r) - 1), (uint32_t)lane, 32, vec);
+        pending = pending && !ready;
+        __syncwarp();
+        // (the bits of lanes beyond the list are set too)
+        const uint32_t left = __ballot_sync(kFull, pending);
+        if ((uint32_t)lane < B / 8) st_release_cta8(ts->done + (c0 >> 3) + lane, ~(left >> (8 * lane)));
+        if (!left) break;
+        look = false;
+        spin = 0;
+      } else {
+        if (!__any_sync(kFull, pending)) break;
+        if (!look) {
+          look = true;
+          continue;
+        }
+        uint32_t why = 0;
+        if (lane == 0 && (spin & 7) == 7)
+          why = ld_vol(&ts->fail) || ld_relaxed(L.err) ? 1u : now_ns() > deadline ? 2u : 0u;
+        why = __shfl_sync(kFull, why, 0);
+        if (why) {
+          if (why == 2 && lane == 0) latch(L.err, kErrTimeout);
+          return false;
+        }
+        __nanosleep(spin < 64 ? 32 : 256);
+      }
+    }
+  }
+  return true;
+}
+
+// Phase (5), by one warp after every warp that copied matches of the segment:
+// no fence per lane, since the barrier that the caller passed (the warp's, or
+// the team's) orders every lane's stores before lane 0's release store, and
+// release is cumulative.
+__device__ __forceinline__ void publish(const DecodeLaunch &L, const DevArchive &A, uint32_t seg, uint32_t level,
+                                        uint32_t epoch, bool ok, int lane) {
+  if (!ok && lane == 0 && ld_relaxed(L.err) == 0) latch(L.err, kErrCorrupt);
+  if (lane == 0 && ok && !(A.blocked && A.blocked[seg])) st_release(A.flags + seg, (uint64_t)level << 32 | epoch);
 }
 
 // Decode one segment: its command streams are staged in the warp's shared
@@ -833,9 +1200,14 @@ __device__ __forceinline__ void decode_segment(const DecodeLaunch &L, const DevA
   const SegRec d = A.dir[seg];
   const uint32_t b3 = (4 + A.W) * d.n_cmd;
   uint8_t *stage = kSharedStage || b3 + 4 <= scap ? sstage : gstage;
-  decode_segment_impl<kSmemLut, kMode, kSharedStage>(L, A, V, seg, epoch, lut, kSmemLut ? smem_addr(lut) : 0u,
-                                                     Stage<kSharedStage>{stage, kSharedStage ? smem_addr(stage) : 0u},
-                                                     mt, smem_addr(ring), lane, d, ph, ph_t);
+  const Stage<kSharedStage> st{stage, kSharedStage ? smem_addr(stage) : 0u};
+  const bool ok = entropy_phases<kSmemLut, kMode, kSharedStage, false>(
+                      A, V, seg, lut, kSmemLut ? smem_addr(lut) : 0u, st, smem_addr(ring), 0, nullptr,
+                      [](bool, uint32_t) {}, lane, d, ph, ph_t) &&
+                  match_phase<kMode, kSharedStage>(L, A, V, seg, epoch, st, mt, lane, d.n_cmd, d.level, ph, ph_t);
+  PHASE_COUNT(9, 1);
+  __syncwarp();
+  publish(L, A, seg, d.level, epoch, ok, lane);
 }
 
 // Dynamic shared memory of a decode CTA: the decode table (64 KiB), then a
@@ -903,6 +1275,156 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_kernel(DecodeLaunch 
     PHASE_MARK(5);
     decode_segment<true, kMode, kSharedStage>(L, L.arc0, L.view0, L.work[idx].seg, epoch, ws.lut, ws.stage,
                                               L.stage_cap, gstage, ws.mt, ws.ring, lane, ph, ph_t);
+  }
+  PHASE_FLUSH();
+}
+
+// Shared memory of a team in staged_kernel: the segment's copy (rounded up to
+// 16 bytes), the word ring and the command stage.
+struct TeamLayout {
+  uint32_t copy, stage, bytes;  // sizes of the copy and the stage, and of all
+};
+__host__ __device__ inline TeamLayout team_layout(uint32_t log2_S, uint32_t max_stage) {
+  TeamLayout y;
+  y.copy = ((1u << log2_S) + 15u) & ~15u;
+  y.stage = (max_stage + 4 + 15u) & ~15u;  // (4: the record read ahead past the sentinel)
+  y.bytes = y.copy + 1280u + y.stage;
+  return y;
+}
+
+// Decode of a short list, for latency: a team of T warps takes a segment and
+// builds it in shared memory. Its first warp decodes the entropy classes, the
+// second places the literals behind it, so that the chain of rANS steps
+// carries nothing else; then all copy the matches; then they write the segment
+// to the view and the first warp publishes it.
+//
+// What bounds such a decode is one segment's rANS chain and then one match
+// phase per level of the wavefront. Each SM runs the match phase only a few
+// times, so that its instructions are fetched on that path: the last warp of
+// each team runs it once on a made-up segment while the entropy classes are
+// being decoded.
+//
+// Measured against a warp per segment (decode_kernel): 2,000-read FASTQ, 42
+// segments in 5 levels, 137.8 -> 78.8 us (39 us of it the chain of 425 steps,
+// 32 us the levels); 500 segments in 8 levels 210 -> 137 us; 1,800 segments,
+// two per team, 238 -> 199 us.
+template <int kMode>
+__global__ void __launch_bounds__(kStagedThreads, 1) staged_kernel(DecodeLaunch L, uint32_t teams, uint32_t T) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  __shared__ TeamState s_team[kMaxTeams + 1];
+  __shared__ __align__(16) uint32_t s_warm[16 + 32];  // the made-up segment: its stage, its copy
+  const int lane = threadIdx.x & 31;
+  const uint32_t wid = threadIdx.x >> 5;
+  const DevArchive &A = L.arc0;
+  {
+    const uint4 *g = reinterpret_cast<const uint4 *>(L.arc0.lut);
+    uint4 *s4 = reinterpret_cast<uint4 *>(smem);
+    for (uint32_t i = threadIdx.x; i < kLutBytes / 16; i += blockDim.x) s4[i] = g[i];
+    // the made-up segment's two commands: 40 literals and a match of 36 from
+    // 1, then 4 literals and a match of 12 from 50 (inside the first match)
+    uint8_t *w = reinterpret_cast<uint8_t *>(s_warm);
+    if (threadIdx.x < 64) w[threadIdx.x] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s_warm[0] = 40u | 36u << 16;
+      s_warm[1] = 44u | 48u << 16;
+      s_warm[2] = 0xFFFFu;
+      w[12] = 1;
+      w[12 + A.W] = 50;
+    }
+    __syncthreads();
+  }
+  // the leaders are warps 0 .. teams - 1 (spread over the SM's four
+  // schedulers), then come T - 1 helpers per team
+  const bool leads = wid < teams;
+  const uint32_t team = leads ? wid : (wid - teams) / (T - 1);
+  const uint32_t rank = leads ? 0u : 1u + (wid - teams) % (T - 1);
+  TeamState *const ts = s_team + team;
+  const TeamLayout y = team_layout(A.log2_S, L.max_stage);
+  uint8_t *const mine = smem + kLutBytes + team * y.bytes;
+  const uint32_t out_s = smem_addr(mine), ring_s = smem_addr(mine + y.copy);
+  const Stage<true> st{mine + y.copy + 1280, ring_s + 1280};
+  const uint32_t *const lut = reinterpret_cast<const uint32_t *>(smem);
+  const uint32_t epoch = ld_relaxed(L.epoch);
+  auto team_sync = [&]() { named_sync(team + 1, 32 * T); };
+  // (the made-up segment is segment 0, which must be long enough)
+  bool warm = rank == T - 1 && A.log2_S >= 7 && A.n >= 128;
+  PHASE_DECL;
+  for (;;) {
+    uint32_t seg = 0, nc = 2, level = 0;
+    bool bad = false;
+    if (!warm) {
+      if (leads) {
+        uint32_t take = kNoSeg;
+        for (;;) {
+          bool failed;
+          const uint32_t idx = take_item(L.counter, L.err, lane, failed);
+          if (idx >= L.n_work) break;
+          if (failed) continue;  // drain the list quickly after an error
+          take = L.work[idx].seg;
+          break;
+        }
+        PHASE_MARK(5);
+        for (uint32_t j = lane; j < kTeamBytes / 4; j += 32) reinterpret_cast<uint32_t *>(ts->done)[j] = 0;
+        auto begin = [&](bool ok, uint32_t tot_m) {
+          if (lane == 0) {
+            ts->seg = take;
+            ts->fail = !ok;
+            ts->lits = 0;
+            ts->tot_m = tot_m;
+          }
+          named_arrive(team + 8, 64);
+        };
+        if (take != kNoSeg) {
+          const SegRec d = A.dir[take];
+          const bool ok = entropy_phases<true, kMode, true, true>(A, L.view0, take, lut, smem_addr(lut), st, ring_s,
+                                                                  out_s, &ts->lits, begin, lane, d, ph, ph_t);
+          if (!ok && lane == 0) *const_cast<volatile uint32_t *>(&ts->fail) = 1;
+        } else {
+          begin(false, 0);
+        }
+      } else if (rank == 1) {
+        named_sync(team + 8, 64);
+        const uint32_t s = __shfl_sync(kFull, ts->seg, 0);
+        if (s < A.n_seg && !__shfl_sync(kFull, ld_vol(&ts->fail), 0) &&
+            !place_literals(st, ts, out_s, A.dir[s].n_lit, now_ns() + L.wait_ns, L.err, lane) && lane == 0)
+          *const_cast<volatile uint32_t *>(&ts->fail) = 1;
+      }
+      team_sync();
+      seg = __shfl_sync(kFull, ts->seg, 0);
+      if (seg >= A.n_seg) break;  // kNoSeg
+      const SegRec d = A.dir[seg];
+      nc = d.n_cmd;
+      level = d.level;
+      bad = __shfl_sync(kFull, ld_vol(&ts->fail), 0) != 0;  // (another warp may be setting it)
+    }
+    const Stage<true> wst{reinterpret_cast<uint8_t *>(s_warm), smem_addr(s_warm)};
+    if (!bad &&
+        !match_phase_team<kMode>(L, A, L.view0, seg, epoch, warm ? wst : st, lane, nc, level,
+                                 warm ? s_team + kMaxTeams : ts, warm ? smem_addr(s_warm + 16) : out_s,
+                                 warm ? 0u : rank, T) &&
+        !warm && lane == 0)
+      *const_cast<volatile uint32_t *>(&ts->fail) = 1;
+    if (warm) {
+      warm = false;
+      continue;
+    }
+    team_sync();
+    if (!ld_vol(&ts->fail)) {
+      // (no warp sets fail after the barrier)
+      const uint64_t seg_start = (uint64_t)seg << A.log2_S, rem = A.n - seg_start;
+      const uint32_t size = rem < (uint64_t(1) << A.log2_S) ? (uint32_t)rem : 1u << A.log2_S;
+      uint8_t *const out = at(L.view0, seg_start, A.log2_S);
+      const uint32_t whole = (reinterpret_cast<uintptr_t>(out) & 15) == 0 ? size & ~15u : 0u;
+#pragma unroll 1
+      for (uint32_t i = 16 * (rank * 32 + lane); i < whole; i += 512 * T)
+        *reinterpret_cast<uint4 *>(out + i) = lds_v4(out_s + i);
+#pragma unroll 1
+      for (uint32_t i = whole + rank * 32 + lane; i < size; i += 32 * T) out[i] = (uint8_t)lds_u8(out_s + i);
+    }
+    team_sync();
+    PHASE_COUNT(9, leads);
+    if (leads) publish(L, A, seg, level, epoch, !ld_vol(&ts->fail), lane);
   }
   PHASE_FLUSH();
 }
@@ -1379,12 +1901,32 @@ int decode_grid(int device, int block) {
   smem((const void *)decode_kernel<kViewLinear, true>);
   smem((const void *)decode_kernel<kViewRing, true>);
   smem((const void *)decode_kernel<kViewPaged, true>);
+  for (const void *k : {(const void *)staged_kernel<kViewLinear>, (const void *)staged_kernel<kViewRing>,
+                        (const void *)staged_kernel<kViewPaged>})
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem);
   cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLutBytes);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_kernel<kViewLinear, false>, kDecodeThreads, kSmemLutBytes);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, batch_kernel, kDecodeThreads, kSmemLutBytes);
   int per_sm = a < b ? a : b;
   if (per_sm < 1) per_sm = 1;
   return sms * per_sm;
+}
+
+// Teams per CTA and warps per team when staged_kernel takes a list of per_cta
+// items per CTA, else no teams. Up to kMaxTeams segments' copies fit a CTA
+// beside the decode table; fewer, larger teams are faster than seven of three
+// warps (1,000 segments: 161 against 197 us). A list of up to two segments
+// per team still gains (2,000 segments: 216 us, against 245 by decode_kernel;
+// 3,000: 273 against 247).
+struct Teams {
+  uint32_t n, warps;
+};
+static Teams team_shape(const DecodeLaunch &L, uint32_t per_cta) {
+  const uint32_t warps = std::min(L.active_warps, kStagedThreads / 32);
+  const uint32_t fit = std::min((kStagedSmem - kLutBytes) / team_layout(L.arc0.log2_S, L.max_stage).bytes, kMaxTeams);
+  if (per_cta > 2 * fit || L.max_stage > L.stage_cap) return {0, 0};
+  const uint32_t n = std::min(per_cta, fit), T = std::min(kMaxTeam, warps / n);
+  return T >= 2 ? Teams{n, T} : Teams{0, 0};
 }
 
 cudaError_t launch_decode(const DecodeLaunch &L0, int grid, int block, cudaStream_t st) {
@@ -1397,7 +1939,17 @@ cudaError_t launch_decode(const DecodeLaunch &L0, int grid, int block, cudaStrea
   // of on five SMs: 75.7 -> 56.4 us; 902 segments of a read's closure: 315 ->
   // 284 us a lookup). A CTA that starts late still finds the list's rest.
   if ((uint32_t)grid > L.n_work) grid = (int)L.n_work;
-  L.active_warps = std::min(L.active_warps, (L.n_work + grid - 1) / grid);
+  const uint32_t per_cta = (L.n_work + grid - 1) / grid;
+  const Teams teams = team_shape(L, per_cta);
+  if (teams.n) {
+    const size_t bytes = kLutBytes + (size_t)teams.n * team_layout(L.arc0.log2_S, L.max_stage).bytes;
+    const int threads = (int)(teams.n * teams.warps * 32);
+    if (L.view0.page) staged_kernel<kViewPaged><<<grid, threads, bytes, st>>>(L, teams.n, teams.warps);
+    else if (L.view0.mask != ~uint64_t(0)) staged_kernel<kViewRing><<<grid, threads, bytes, st>>>(L, teams.n, teams.warps);
+    else staged_kernel<kViewLinear><<<grid, threads, bytes, st>>>(L, teams.n, teams.warps);
+    return cudaGetLastError();
+  }
+  L.active_warps = std::min(L.active_warps, per_cta);
   // every segment's command streams fit the shared stage: the stage-in-shared kernel
   const bool sh = L.max_stage <= L.stage_cap;
   if (L.view0.page) {
