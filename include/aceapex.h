@@ -301,15 +301,14 @@ int aceapex_server_get_stats(aceapex_server *s, aceapex_server_stats *out);
  * queued on `stream` has run. The header (128 bytes) is read to the host
  * first, so the call synchronises `stream` once before queuing the decode.
  *
- * Scratch: a fixed array of about 4.6 MiB in the library's device memory,
+ * Scratch: a fixed array of about 1.1 MiB in the library's device memory,
  * which every GPU that loads the library holds until the process exits. The
  * first call on a device looks up the array's device address (with that
  * device current). Archives
  * of more than 65,536 segments (1 GiB at 16 KiB segments) are rejected with
  * ERANGE. All calls share the array and it keeps the last call's contents;
  * each call resets what must start at zero, but calls that overlap on the
- * GPU race and must not be issued. The decode uses 256 warps, so it is
- * slower than aceapex_decode_all. Errors: EINVAL (null, misaligned or short
+ * GPU race and must not be issued. Errors: EINVAL (null, misaligned or short
  * archive), ECORRUPT (bad header), ERANGE (too many segments, out_cap < N),
  * ECUDA.
  */

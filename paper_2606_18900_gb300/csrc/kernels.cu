@@ -1316,6 +1316,7 @@ __global__ void __launch_bounds__(kStagedThreads, 1) staged_kernel(DecodeLaunch 
   const int lane = threadIdx.x & 31;
   const uint32_t wid = threadIdx.x >> 5;
   const DevArchive &A = L.arc0;
+  if (L.stage_need && ld_relaxed(L.stage_need) > L.max_stage) return;  // (another kernel takes the list)
   {
     const uint4 *g = reinterpret_cast<const uint4 *>(L.arc0.lut);
     uint4 *s4 = reinterpret_cast<uint4 *>(smem);
@@ -2157,109 +2158,191 @@ cudaError_t launch_window_crc(OutView v, uint64_t lo, uint64_t hi, uint64_t wind
 // library holds until the process exits.
 //
 // Limits: at most kNoAllocMaxSegments segments (1 GiB of output at 16 KiB
-// segments); larger archives are rejected with ACEAPEX_ERANGE. The decode
-// runs on kNoAllocWarps warps only, so it is slower than
-// aceapex_decode_all. All calls share the array and it keeps the last
+// segments); larger archives are rejected with ACEAPEX_ERANGE. All calls share the array and it keeps the last
 // call's contents: each call clears the words that must start at zero and
 // takes a fresh epoch, but calls that overlap on the GPU (on different
 // streams, or from different threads) race and must not be issued.
 namespace {
 
 constexpr uint32_t kNoAllocMaxSegments = 65536;
-constexpr uint32_t kNoAllocWarps = 256;
-constexpr size_t kNoAllocCtlBytes = 256;                       // counter, epoch, err
+constexpr size_t kNoAllocCtlBytes = 4096;                      // control words
 constexpr size_t kNoAllocLutBytes = 4 * kScale * sizeof(uint32_t);
 constexpr size_t kNoAllocFlagBytes = kNoAllocMaxSegments * sizeof(uint64_t);
-constexpr size_t kNoAllocStageBytes = (size_t)kNoAllocWarps * kStageBytes;
-constexpr size_t kNoAllocBytes = kNoAllocCtlBytes + kNoAllocLutBytes + kNoAllocFlagBytes + kNoAllocStageBytes;
+constexpr size_t kNoAllocWorkBytes = kNoAllocMaxSegments * sizeof(WorkItem);
+constexpr size_t kNoAllocBytes = kNoAllocCtlBytes + kNoAllocLutBytes + kNoAllocFlagBytes + kNoAllocWorkBytes;
 
-// about 4.3 MiB per device
+// about 1.1 MiB per device
 static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocBytes];
 
-// control words at the start of the array
-constexpr size_t kCtlCounter = 0, kCtlEpoch = 4, kCtlErr = 8, kCtlEmpty = 12;
+// control words at the start of the array: the work counter, the epoch, the
+// error word, the classes without symbols (a bit each), the largest command
+// stage of any segment, and per level the number of segments and the next
+// place in the work list less the level's start
+struct NoAllocCtl {
+  uint32_t counter, epoch, err, empty, need, pad[3];
+  uint32_t hist[256], next[256];
+};
+static_assert(sizeof(NoAllocCtl) <= kNoAllocCtlBytes, "the control words fit their part of the array");
 
-// builds the decode table from the archive's tables, checks their sums,
-// clears the counter and the error word, and takes the next epoch
-__global__ void noalloc_setup_kernel(const uint8_t *tables) {
-  uint8_t *base = g_noalloc_scratch;
-  uint32_t *ctl = reinterpret_cast<uint32_t *>(base);
-  uint32_t *lut = reinterpret_cast<uint32_t *>(base + kNoAllocCtlBytes);
-  __shared__ uint32_t cum[4][257];
-  __shared__ uint32_t bad;
-  __shared__ uint32_t empty;
-  if (threadIdx.x == 0) {
-    bad = 0;
-    empty = 0;
-    for (int c = 0; c < 4; ++c) {
-      uint32_t s = 0;
-      cum[c][0] = 0;
-      for (int x = 0; x < 256; ++x) {
-        s += (uint32_t)tables[512 * c + 2 * x] | ((uint32_t)tables[512 * c + 2 * x + 1] << 8);
-        cum[c][x + 1] = s;
-      }
-      if (s != 0 && s != kScale) bad = 1;
-      if (s == 0) empty |= 1u << c;
-    }
-  }
+constexpr uint32_t kNoAllocThreads = 1024;
+
+// Builds the decode table from the archive's tables, checks their sums,
+// clears the control words and takes the next epoch. One CTA: a thread per
+// table entry for the prefix sums, then a thread per table slot, which finds
+// its symbol by binary search (one thread summing 1,024 entries and writing
+// runs of slots took 54 us; this takes 6).
+__global__ void __launch_bounds__(kNoAllocThreads) noalloc_setup_kernel(const uint8_t *tables) {
+  NoAllocCtl *ctl = reinterpret_cast<NoAllocCtl *>(g_noalloc_scratch);
+  uint32_t *lut = reinterpret_cast<uint32_t *>(g_noalloc_scratch + kNoAllocCtlBytes);
+  __shared__ uint32_t cum[4][257];  // cum[c][x + 1]: frequencies of symbols 0 .. x
+  __shared__ uint32_t wsum[32], total[4];
+  const uint32_t tid = threadIdx.x, c = tid >> 8, x = tid & 255, lane = tid & 31, w = tid >> 5;
+  const uint32_t f = (uint32_t)tables[2 * tid] | (uint32_t)tables[2 * tid + 1] << 8;
+  const uint32_t incl = warp_incl_scan(f, (int)lane);
+  if (lane == 31) wsum[w] = incl;
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < 4 * 256; i += blockDim.x) {
-    const uint32_t c = i >> 8, x = i & 255, f = cum[c][x + 1] - cum[c][x];
-    for (uint32_t k = 0; k < f && !bad; ++k) lut[c * kScale + cum[c][x] + k] = x | (k << 8) | ((f - 1) << 20);
+  uint32_t before = 0;
+  for (uint32_t v = w & ~7u; v < w; ++v) before += wsum[v];
+  cum[c][x + 1] = before + incl;
+  if (x == 0) cum[c][0] = 0;
+  if (x == 255) total[c] = before + incl;
+  for (uint32_t i = tid; i < 256; i += kNoAllocThreads) ctl->hist[i] = ctl->next[i] = 0;
+  __syncthreads();
+  const bool bad = (total[0] && total[0] != kScale) || (total[1] && total[1] != kScale) ||
+                   (total[2] && total[2] != kScale) || (total[3] && total[3] != kScale);
+  for (uint32_t i = tid; i < 4 * kScale && !bad; i += kNoAllocThreads) {
+    const uint32_t cl = i >> kScaleBits, slot = i & (kScale - 1);
+    if (!total[cl]) {
+      lut[i] = 0;
+      continue;
+    }
+    uint32_t s = 0;  // the symbol with cum <= slot < cum + f: the number of later starts at or below slot
+    for (uint32_t d = 128; d; d >>= 1)
+      if (cum[cl][s + d] <= slot) s += d;
+    lut[i] = s | (slot - cum[cl][s]) << 8 | (cum[cl][s + 1] - cum[cl][s] - 1) << 20;
   }
-  if (threadIdx.x == 0) {
-    ctl[kCtlCounter / 4] = 0;
-    ctl[kCtlErr / 4] = bad ? kErrCorrupt : 0u;
-    ctl[kCtlEmpty / 4] = empty;
-    ctl[kCtlEpoch / 4] = ctl[kCtlEpoch / 4] + 1u;
+  if (tid == 0) {
+    ctl->counter = 0;
+    ctl->err = bad ? kErrCorrupt : 0u;
+    ctl->empty = (total[0] ? 0u : 1u) | (total[1] ? 0u : 2u) | (total[2] ? 0u : 4u) | (total[3] ? 0u : 8u);
+    ctl->need = 0;
+    ctl->epoch = ctl->epoch + 1u;
   }
 }
 
-// segments in index order (every source segment precedes its reader, so a
-// warp only waits for segments that running warps took earlier)
-__global__ void __launch_bounds__(256) noalloc_decode_kernel(DecodeLaunch L, uint64_t payload_bytes,
-                                                             uint32_t max_level) {
-  const int lane = threadIdx.x & 31;
-  const uint32_t gwarp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (gwarp >= kNoAllocWarps) return;
-  uint8_t *stage = g_noalloc_scratch + kNoAllocCtlBytes + kNoAllocLutBytes + kNoAllocFlagBytes +
-                   (size_t)gwarp * kStageBytes;
-  __shared__ MatchTable mts[8];
-  __shared__ __align__(16) uint16_t rings_raw[8][640];
-  uint16_t *ring = rings_raw[threadIdx.x >> 5];
-  const uint32_t epoch = ld_relaxed(L.epoch);
-  PHASE_DECL;
-  const uint32_t empty = reinterpret_cast<const uint32_t *>(g_noalloc_scratch)[kCtlEmpty / 4];
-  const DevArchive &A = L.arc0;
-  for (;;) {
-    bool failed;
-    const uint32_t seg = take_item(L.counter, L.err, lane, failed);
-    if (seg >= A.n_seg) break;
-    if (failed) continue;
-    // the directory was not validated on the host: check what the shared
-    // segment decoder relies on before calling it
-    const SegRec d = A.dir[seg];
+// A thread per segment: checks what the decoder relies on in its directory
+// record (which was not validated on the host), sets its flag word, and counts
+// the segments per level and the largest command stage.
+__global__ void __launch_bounds__(kNoAllocThreads) noalloc_scan_kernel(DevArchive A, uint64_t payload_bytes,
+                                                                       uint32_t max_level) {
+  NoAllocCtl *ctl = reinterpret_cast<NoAllocCtl *>(g_noalloc_scratch);
+  __shared__ uint32_t hist[256], need;
+  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
+  if (threadIdx.x == 0) need = 0;
+  __syncthreads();
+  const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s < A.n_seg) {
+    const SegRec d = A.dir[s];
+    const uint32_t empty = ctl->empty;
     // (the payload test is written so that no sum can wrap)
     const uint64_t n_sym = (uint64_t)d.n_cmd * (4 + A.W) + d.n_lit;
     const bool sane = n_sym <= kMaxSym && (d.payload_off & 15) == 0 && d.payload_off <= payload_bytes &&
                       payload_bytes - d.payload_off >= 128 &&
                       d.n_words <= (payload_bytes - d.payload_off - 128) / 2 && d.level <= max_level &&
                       !(d.n_cmd && (empty & 7u)) && !(d.n_lit && (empty & 8u));
-    if (!sane) {
-      if (lane == 0) latch(L.err, kErrCorrupt);
-      continue;
-    }
-    decode_segment<false, kViewLinear, false>(L, A, L.view0, seg, epoch, A.lut, stage, 0, stage,
-                                              &mts[threadIdx.x >> 5], ring, lane, ph, ph_t);
+    if (!sane) latch(&ctl->err, kErrCorrupt);  // no segment is decoded then
+    else atomicMax(&need, d.n_cmd * (4 + A.W) + 4);
+    A.flags[s] = (uint64_t)d.level << 32;
+    atomicAdd(&hist[min((uint32_t)d.level, 255u)], 1u);
   }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x)
+    if (hist[i]) atomicAdd(&ctl->hist[i], hist[i]);
+  if (threadIdx.x == 0 && need) atomicMax(&ctl->need, need);
+}
+
+// The work list in level order (any order within a level): each CTA reserves
+// its segments' places of a level with one atomic.
+__global__ void __launch_bounds__(kNoAllocThreads) noalloc_order_kernel(DevArchive A, WorkItem *work) {
+  NoAllocCtl *ctl = reinterpret_cast<NoAllocCtl *>(g_noalloc_scratch);
+  __shared__ uint32_t start[256], count[256], wsum[8];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  uint32_t h = 0, incl = 0;
+  if (tid < 256) {
+    count[tid] = 0;
+    h = ctl->hist[tid];
+    incl = warp_incl_scan(h, (int)lane);
+    if (lane == 31) wsum[w] = incl;
+  }
+  __syncthreads();
+  const uint32_t s = blockIdx.x * blockDim.x + tid;
+  uint32_t lv = 0, at = 0;
+  if (s < A.n_seg) {
+    lv = min((uint32_t)A.dir[s].level, 255u);
+    at = atomicAdd(&count[lv], 1u);
+  }
+  __syncthreads();
+  if (tid < 256) {
+    uint32_t before = 0;
+    for (uint32_t v = 0; v < w; ++v) before += wsum[v];
+    start[tid] = before + incl - h + (count[tid] ? atomicAdd(&ctl->next[tid], count[tid]) : 0u);
+  }
+  __syncthreads();
+  if (s < A.n_seg) work[start[lv] + at] = WorkItem{0u, s};
+}
+
+// Warps of a CTA, and bytes of shared command stage each: 32 with the usual
+// stage when every segment of the archive fits it, else 8 with the largest
+// stage that a segment can have.
+constexpr uint32_t kNoAllocBigWarps = 8;
+static_assert(kLutBytes + kNoAllocBigWarps * (1280 + sizeof(MatchTable) + kStageBytes) <=
+                  kLutBytes + (kDecodeThreads / 32) * (1280 + sizeof(MatchTable) + kSmemStage),
+              "both splits of the shared memory fit the launch");
+
+// The whole chip, a warp per segment, in level order. (256 warps on 32 SMs,
+// with the tables and the command stages in global memory and in index order,
+// took 3.06 ms for 64 MiB of FASTQ.)
+__global__ void __launch_bounds__(kDecodeThreads, 1) noalloc_decode_kernel(DecodeLaunch L, bool small_done) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const NoAllocCtl *ctl = reinterpret_cast<const NoAllocCtl *>(g_noalloc_scratch);
+  const bool big = ctl->need > kSmemStage;
+  if (small_done && !big) return;  // staged_kernel has decoded the list
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  {
+    const uint4 *g = reinterpret_cast<const uint4 *>(L.arc0.lut);
+    uint4 *s4 = reinterpret_cast<uint4 *>(smem);
+    for (uint32_t i = threadIdx.x; i < kLutBytes / 16; i += blockDim.x) s4[i] = g[i];
+    __syncthreads();
+  }
+  const uint32_t warps = big ? kNoAllocBigWarps : kDecodeThreads / 32;
+  if ((uint32_t)wid >= min(warps, L.active_warps)) return;
+  uint8_t *rings = smem + kLutBytes;
+  uint16_t *ring = reinterpret_cast<uint16_t *>(rings + wid * 1280);
+  MatchTable *mt = reinterpret_cast<MatchTable *>(rings + warps * 1280) + wid;
+  uint8_t *stage = rings + warps * (1280 + sizeof(MatchTable)) + (size_t)wid * (big ? kStageBytes : kSmemStage);
+  const uint32_t epoch = ld_relaxed(L.epoch);
+  PHASE_DECL;
+  for (;;) {
+    bool failed;
+    const uint32_t idx = take_item(L.counter, L.err, lane, failed);
+    if (idx >= L.n_work) break;
+    if (failed) continue;
+    decode_segment<true, kViewLinear, true>(L, L.arc0, L.view0, L.work[idx].seg, epoch,
+                                            reinterpret_cast<const uint32_t *>(smem), stage, kStageBytes, nullptr, mt,
+                                            ring, lane, ph, ph_t);
+  }
+  PHASE_FLUSH();
 }
 
 __global__ void noalloc_status_kernel(uint32_t *status) {
-  *status = reinterpret_cast<const uint32_t *>(g_noalloc_scratch)[kCtlErr / 4];
+  *status = reinterpret_cast<const NoAllocCtl *>(g_noalloc_scratch)->err;
 }
 
 std::mutex g_noalloc_mu;
-uint8_t *g_noalloc_addr[64] = {};
+struct NoAllocDevice {
+  uint8_t *base = nullptr;  // device address of the scratch array
+  int sms = 0;
+} g_noalloc_dev[64];
 
 }  // namespace
 
@@ -2271,16 +2354,26 @@ extern "C" int aceapex_decode_all_noalloc(const void *d_archive, uint64_t nbytes
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 4;  // ACEAPEX_ECUDA
   // set-up, once per device with that device current: the device address of
-  // the scratch array (its name in host code is only a stand-in)
+  // the scratch array (its name in host code is only a stand-in) and the
+  // kernels' shared-memory limits
   uint8_t *base = nullptr;
+  int grid = 0;
   {
     std::lock_guard<std::mutex> lk(g_noalloc_mu);
-    if (!g_noalloc_addr[dev]) {
+    NoAllocDevice &D = g_noalloc_dev[dev];
+    if (!D.base) {
       void *p = nullptr;
-      if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return 4;
-      g_noalloc_addr[dev] = static_cast<uint8_t *>(p);
+      if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p ||
+          cudaDeviceGetAttribute(&D.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+          cudaFuncSetAttribute(noalloc_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kSmemLutBytes) != cudaSuccess ||
+          cudaFuncSetAttribute(staged_kernel<kViewLinear>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kStagedSmem) != cudaSuccess)
+        return 4;
+      D.base = static_cast<uint8_t *>(p);
     }
-    base = g_noalloc_addr[dev];
+    base = D.base;
+    grid = D.sms;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the header, read into host stack memory
@@ -2329,17 +2422,34 @@ extern "C" int aceapex_decode_all_noalloc(const void *d_archive, uint64_t nbytes
   L.view0.base = static_cast<uint8_t *>(d_out);
   L.view0.origin = 0;
   L.view0.mask = ~uint64_t(0);
-  L.counter = reinterpret_cast<uint32_t *>(base + kCtlCounter);
-  L.epoch = reinterpret_cast<const uint32_t *>(base + kCtlEpoch);
-  L.err = reinterpret_cast<uint32_t *>(base + kCtlErr);
+  NoAllocCtl *ctl = reinterpret_cast<NoAllocCtl *>(base);
+  WorkItem *work = reinterpret_cast<WorkItem *>(base + kNoAllocCtlBytes + kNoAllocLutBytes + kNoAllocFlagBytes);
+  L.counter = &ctl->counter;
+  L.epoch = &ctl->epoch;
+  L.err = &ctl->err;
+  L.work = work;
+  L.n_work = (uint32_t)n_seg;
   L.scratch = nullptr;
-  L.scratch_warps = kNoAllocWarps;
   L.wait_ns = 2000000000ull;
-  noalloc_setup_kernel<<<1, 256, 0, st>>>(arc + kHeaderBytes);
-  // (a corrupt record's level is caught by that segment's own checks, and a
-  // reader that waits for it gives up once that segment latches the error)
-  launch_init_flags(A.flags, A.dir, n_seg, st);
-  noalloc_decode_kernel<<<kNoAllocWarps / 8, 256, 0, st>>>(L, payload_bytes, h[30]);
+  L.active_warps = kDecodeThreads / 32;
+  L.stage_cap = L.max_stage = kSmemStage;
+  L.stage_need = &ctl->need;
+  const unsigned blocks = (unsigned)((n_seg + kNoAllocThreads - 1) / kNoAllocThreads);
+  noalloc_setup_kernel<<<1, kNoAllocThreads, 0, st>>>(arc + kHeaderBytes);
+  // (a reader that waits for a segment whose record is corrupt gives up: the
+  // error is latched before any segment is taken)
+  noalloc_scan_kernel<<<blocks, kNoAllocThreads, 0, st>>>(A, payload_bytes, h[30]);
+  noalloc_order_kernel<<<blocks, kNoAllocThreads, 0, st>>>(A, work);
+  // as launch_decode: spread a short list, and give it teams
+  if ((uint64_t)grid > n_seg) grid = (int)n_seg;
+  const uint32_t per_cta = (L.n_work + grid - 1) / grid;
+  const Teams teams = team_shape(L, per_cta);
+  if (teams.n) {
+    const size_t bytes = kLutBytes + (size_t)teams.n * team_layout(log2_S, L.max_stage).bytes;
+    staged_kernel<kViewLinear><<<grid, (int)(teams.n * teams.warps * 32), bytes, st>>>(L, teams.n, teams.warps);
+  }
+  L.active_warps = std::min(L.active_warps, per_cta);
+  noalloc_decode_kernel<<<grid, kDecodeThreads, kSmemLutBytes, st>>>(L, teams.n != 0);
   noalloc_status_kernel<<<1, 1, 0, st>>>(d_status);
   return cudaGetLastError() == cudaSuccess ? 0 : 4;
 }

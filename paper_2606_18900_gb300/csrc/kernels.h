@@ -58,6 +58,8 @@ struct DecodeLaunch {
   uint32_t active_warps;    // warps per CTA that take work (<= kDecodeThreads / 32)
   uint32_t stage_cap;       // bytes of a warp's shared staging to use (<= kSmemStage)
   uint32_t max_stage;       // largest command stage (bytes) of any segment the launch may decode
+  const uint32_t *stage_need;  // when not null: a device word with the list's largest command stage, found on the
+                               // device; staged_kernel leaves the list alone when it exceeds max_stage
 };
 
 // command stage of a segment: its n_cmd * (4 + W) command symbols plus a
