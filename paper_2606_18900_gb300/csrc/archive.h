@@ -180,6 +180,8 @@ struct aceapex_archive {
   DBuf<uint8_t> d_fq_streams;
   DBuf<uint32_t> d_fq_counts, d_fq_nl;
   DBuf<uint64_t> d_fq_offs;
+  cudaStream_t fq_st[3] = {};  // decode parts 1 .. 3; events: start, parts 1 .. 3
+  cudaEvent_t fq_ev[4] = {};
 
   uint32_t *err() const { return d_words.p; }
   uint32_t *epoch() const { return d_words.p + 1; }
@@ -224,6 +226,14 @@ struct aceapex_archive {
     win_ev.clear();
     if (copy_st) cudaStreamDestroy(copy_st);
     copy_st = nullptr;
+    for (cudaEvent_t &e : fq_ev) {
+      if (e) cudaEventDestroy(e);
+      e = nullptr;
+    }
+    for (cudaStream_t &s : fq_st) {
+      if (s) cudaStreamDestroy(s);
+      s = nullptr;
+    }
     stage_work.release();
     stage_batch.release();
   }

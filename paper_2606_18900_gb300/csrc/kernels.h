@@ -129,10 +129,10 @@ struct GatherJob {
 cudaError_t launch_multi_gather(const GatherJob *jobs, uint32_t n_jobs, uint64_t n_chunks, cudaStream_t st);
 
 // Reassembles a FASTQ from its four decoded line streams (base[k], len[k]
-// bytes): newline index of each stream (counts: one u32 per 64 KiB chunk of
-// the longest stream; offs: chunks + 1 u64 per stream; nl[k]: cap[k] u32
-// positions, err latched beyond), then one warp per record copies its four
-// lines to out.
+// bytes; base[k] 16-byte aligned, readable to the next multiple of 16): newline
+// index of each stream (counts: one u32 per 64 KiB chunk of every stream;
+// offs: chunks + 1 u64 per stream; nl[k]: cap[k] u32 positions, err latched
+// beyond), then the lines are copied to out, eight records to a warp.
 cudaError_t launch_fastq_interleave(const uint8_t *const base[4], const uint64_t len[4], uint32_t *counts,
                                     uint64_t *offs, uint32_t *const nl[4], const uint64_t cap[4], uint32_t *err,
                                     uint8_t *out, cudaStream_t st);
