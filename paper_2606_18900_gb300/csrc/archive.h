@@ -158,7 +158,7 @@ struct aceapex_archive {
 
   // ring streaming
   DBuf<uint8_t> d_ring;
-  DBuf<uint32_t> d_seg_crc;
+  DBuf<uint32_t> d_crc_sums;  // zero between windows
   // batch
   std::vector<uint8_t> batch_desc;  // host copy of what d_batch_arcs / d_batch_views hold
   DBuf<DevArchive> d_batch_arcs;
@@ -217,7 +217,7 @@ struct aceapex_archive {
     end_upload();
     d_payload.release(); d_dir.release(); d_lut.release(); d_flags.release(); d_order.release();
     d_words.release(); d_blocked.release(); d_scratch.release(); d_page.release(); d_arena.release();
-    d_work.release(); d_ring.release(); d_seg_crc.release(); d_batch_arcs.release(); d_batch_views.release();
+    d_work.release(); d_ring.release(); d_crc_sums.release(); d_batch_arcs.release(); d_batch_views.release();
     d_fq_streams.release(); d_fq_counts.release(); d_fq_nl.release(); d_fq_offs.release();
     d_host_out.release(); d_win_work.release();
     d_dep_ptr.release(); d_deps.release(); d_cmark.release(); d_clist.release(); d_ccnt.release();

@@ -1017,10 +1017,9 @@ int aceapex_stream_range(aceapex_archive *a, uint64_t lo, uint64_t hi, uint64_t 
     cudaStreamSynchronize(st);
     if (a->d_ring.alloc(ring_bytes) != cudaSuccess) return ACEAPEX_ENOMEM;
   }
-  const uint64_t seg_per_win = window / S + 1;
-  if (a->d_seg_crc.n < seg_per_win) {
-    cudaStreamSynchronize(st);
-    if (a->d_seg_crc.alloc(seg_per_win) != cudaSuccess) return ACEAPEX_ENOMEM;
+  if (!a->d_crc_sums.p) {
+    if (a->d_crc_sums.alloc(2) != cudaSuccess) return ACEAPEX_ENOMEM;
+    if (cudaMemsetAsync(a->d_crc_sums.p, 0, 8, st) != cudaSuccess) return ACEAPEX_ECUDA;
   }
   OutView ring{};
   ring.base = a->d_ring.p;
@@ -1078,7 +1077,7 @@ int aceapex_stream_range(aceapex_archive *a, uint64_t lo, uint64_t hi, uint64_t 
     L.work = a->d_work.p + wstart[k];
     L.n_work = (uint32_t)(wstart[k + 1] - wstart[k]);
     if ((e = launch_decode(L, a->grid, kBlock, st)) != cudaSuccess) return ACEAPEX_ECUDA;
-    if ((e = launch_window_crc(ring, wa, wb, window, d_crc + k, a->d_seg_crc.p, h.log2_S, st)) != cudaSuccess)
+    if ((e = launch_window_crc(ring, wa, wb, d_crc + k, a->d_crc_sums.p, h.log2_S, st)) != cudaSuccess)
       return ACEAPEX_ECUDA;
   }
   return ACEAPEX_OK;

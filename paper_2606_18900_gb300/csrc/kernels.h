@@ -159,8 +159,9 @@ cudaError_t launch_closure_expand(ClosureDev C, uint32_t level, uint32_t gen, cu
 // members sorted by level into work[0 .. n), page[seg] = its position, n into *n_out
 cudaError_t launch_closure_order(ClosureDev C, WorkItem *work, uint32_t *page, uint32_t *n_out, cudaStream_t st);
 
-// CRC-32 of each window [lo + k*window, ...) of the ring view, written to crc[k].
-cudaError_t launch_window_crc(OutView v, uint64_t lo, uint64_t hi, uint64_t window, uint32_t *crc, uint32_t *seg_crc,
-                              uint32_t log2_S, cudaStream_t st);
+// CRC-32 of [lo, hi) of the ring view, written to *crc; sums: two device words
+// that are zero between launches.
+cudaError_t launch_window_crc(OutView v, uint64_t lo, uint64_t hi, uint32_t *crc, uint32_t *sums, uint32_t log2_S,
+                              cudaStream_t st);
 
 }  // namespace aceapex
