@@ -1519,10 +1519,39 @@ __global__ void copy_view_kernel(OutView src, OutView dst, uint32_t log2_S, uint
   }
 }
 
-__global__ void gather_kernel(OutView v, uint32_t log2_S, uint64_t lo, uint64_t n, uint8_t *dst) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+// Bytes [a, b) of dst (absent pages: zeros), by one thread: what of [lo, lo + n)
+// falls into one of dst's aligned 16-byte blocks. One page lookup and one
+// 16-byte store per block (built from two aligned source blocks) when the
+// block's source lies in one segment of at least 16 bytes, aligned in memory.
+__device__ __forceinline__ void gather_block(const OutView &v, uint32_t log2_S, uint64_t lo, uint8_t *dst, uint64_t a,
+                                             uint64_t b) {
+  if (b - a == 16 && log2_S >= 4 && v.page && (reinterpret_cast<uintptr_t>(v.slot_base) & 15) == 0 &&
+      (lo + a) >> log2_S == (lo + b - 1) >> log2_S) {
+    const uint8_t *p = at(v, lo + a, log2_S);
+    uint32_t r[4] = {0, 0, 0, 0};
+    if (p) {
+      const uint32_t dl = (uint32_t)reinterpret_cast<uintptr_t>(p) & 15u;
+      const uint4 *q = reinterpret_cast<const uint4 *>(p - dl);
+      realign16(q[0], dl ? q[1] : make_uint4(0, 0, 0, 0), dl, r);
+    }
+    *reinterpret_cast<uint4 *>(dst + a) = make_uint4(r[0], r[1], r[2], r[3]);
+    return;
+  }
+  for (uint64_t i = a; i < b; ++i) {
     const uint8_t *p = at(v, lo + i, log2_S);
     dst[i] = p ? *p : 0;
+  }
+}
+
+// [lo, lo + n) of the view into dst (any alignment): a thread per aligned
+// 16-byte block of dst (a byte per thread took 25 us for 9.4 MB).
+__global__ void gather_kernel(OutView v, uint32_t log2_S, uint64_t lo, uint64_t n, uint8_t *dst) {
+  const uint64_t off = reinterpret_cast<uintptr_t>(dst) & 15;  // dst's place in its first block
+  const uint64_t blocks = (off + n + 15) >> 4;
+  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < blocks;
+       k += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t a = k ? 16 * k - off : 0, b = min(n, 16 * (k + 1) - off);
+    gather_block(v, log2_S, lo, dst, a, b);
   }
 }
 
@@ -1550,10 +1579,10 @@ __global__ void multi_gather_kernel(const GatherJob *jobs, uint32_t n_jobs, uint
     }
     const GatherJob &J = jobs[lo];
     const uint64_t a = (c - J.chunk0) * kGatherChunk, b = min(J.n, a + kGatherChunk);
-    for (uint64_t i = a + threadIdx.x; i < b; i += blockDim.x) {
-      const uint8_t *p = at(J.v, J.lo + i, J.log2_S);
-      J.dst[i] = p ? *p : 0;
-    }
+    // as gather_kernel: a thread per aligned 16-byte block of dst
+    const uint64_t off = reinterpret_cast<uintptr_t>(J.dst + a) & 15, blocks = (off + (b - a) + 15) >> 4;
+    for (uint64_t k = threadIdx.x; k < blocks; k += blockDim.x)
+      gather_block(J.v, J.log2_S, J.lo, J.dst, k ? a + 16 * k - off : a, min(b, a + 16 * (k + 1) - off));
   }
 }
 
@@ -2080,8 +2109,8 @@ cudaError_t launch_copy_view(OutView src, OutView dst, uint32_t log2_S, uint64_t
 
 cudaError_t launch_gather(OutView v, uint32_t log2_S, uint64_t lo, uint64_t hi, uint8_t *dst, cudaStream_t st) {
   if (hi <= lo) return cudaSuccess;
-  uint64_t n = hi - lo;
-  int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
+  const uint64_t n = hi - lo, want = (n / 16 + 2 + 255) / 256;  // (up to two partial blocks)
+  const int grid = (int)(want < 4096 ? want : 4096);
   gather_kernel<<<grid, 256, 0, st>>>(v, log2_S, lo, n, dst);
   return cudaGetLastError();
 }
