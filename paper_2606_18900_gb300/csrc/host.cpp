@@ -1195,7 +1195,7 @@ int aceapex_decode_fastq_streams(aceapex_archive *const *parts, void *d_out, uin
   }
   // The parts decode side by side, each with its own persistent launch on a
   // share of the SMs in proportion to its rANS symbols and commands (a
-  // command costs about as much as 65 symbols; one
+  // command costs about as much as 85 symbols; one
   // after the other, each would end in its own wavefront and last wave:
   // 745 us for 192 MiB against 390 in all); part 0 on the caller's stream, the others
   // on streams of the handle that start after it and that it waits for. A
@@ -1206,7 +1206,7 @@ int aceapex_decode_fastq_streams(aceapex_archive *const *parts, void *d_out, uin
   for (int k = 0; k < 4; ++k) {
     for (int j = 0; j < k; ++j) apart = apart && parts[j] != parts[k];
     const aceapex_stats &s = parts[k]->stats;
-    all += cost[k] = s.literal_bytes + s.n_commands * (4 + s.W + 60) + 1;
+    all += cost[k] = s.literal_bytes + s.n_commands * (4 + s.W + 80) + 1;
   }
   int rc = ensure_scratch(A);
   if (rc) return rc;
