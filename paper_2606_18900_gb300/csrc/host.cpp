@@ -510,17 +510,24 @@ int decode_closure(aceapex_archive *A, uint64_t s_lo, uint64_t s_hi, cudaStream_
     cudaStreamSynchronize(st);
     if (A->d_work.alloc(std::max<uint64_t>(work.size(), 1024)) != cudaSuccess) return ACEAPEX_ENOMEM;
   }
-  if (A->stage_work.reserve(work.size() * sizeof(WorkItem)) != cudaSuccess) return ACEAPEX_ENOMEM;
-  std::memcpy(A->stage_work.p, work.data(), work.size() * sizeof(WorkItem));
-  cudaError_t e = cudaMemcpyAsync(A->d_work.p, A->stage_work.p, work.size() * sizeof(WorkItem),
-                                  cudaMemcpyHostToDevice, st);
-  A->stage_work.mark(st);
-  if (e != cudaSuccess) return ACEAPEX_ECUDA;
-  if ((e = launch_set_pages(A->d_page.p, A->d_work.p, (uint32_t)work.size(), st)) != cudaSuccess) return ACEAPEX_ECUDA;
   uint32_t *ge = global_epoch(A->device);
   if (!ge) return ACEAPEX_ECUDA;
-  if (begin && (e = launch_begin(ge, A->epoch(), A->counter(), st)) != cudaSuccess) return ACEAPEX_ECUDA;
-  if (!begin && (e = cudaMemsetAsync(A->counter(), 0, 4, st)) != cudaSuccess) return ACEAPEX_ECUDA;
+  cudaError_t e = cudaSuccess;
+  if (begin && work.size() <= kListMax) {
+    WorkList list;
+    list.n = (uint32_t)work.size();
+    for (uint32_t i = 0; i < list.n; ++i) list.seg[i] = work[i].seg;
+    e = launch_begin_list(list, A->d_work.p, A->d_page.p, ge, A->epoch(), A->counter(), st);
+  } else {
+    if (A->stage_work.reserve(work.size() * sizeof(WorkItem)) != cudaSuccess) return ACEAPEX_ENOMEM;
+    std::memcpy(A->stage_work.p, work.data(), work.size() * sizeof(WorkItem));
+    e = cudaMemcpyAsync(A->d_work.p, A->stage_work.p, work.size() * sizeof(WorkItem), cudaMemcpyHostToDevice, st);
+    A->stage_work.mark(st);
+    if (e == cudaSuccess) e = launch_set_pages(A->d_page.p, A->d_work.p, (uint32_t)work.size(), st);
+    if (e == cudaSuccess)
+      e = begin ? launch_begin(ge, A->epoch(), A->counter(), st) : cudaMemsetAsync(A->counter(), 0, 4, st);
+  }
+  if (e != cudaSuccess) return ACEAPEX_ECUDA;
   DecodeLaunch L = base_launch(A);
   OutView v{};
   v.page = A->d_page.p;
@@ -872,9 +879,7 @@ int aceapex_decode_range(aceapex_archive *a, uint64_t lo, uint64_t hi, void *d_o
   uint32_t n = 0;
   rc = decode_closure(a, lo >> a->h.log2_S, (hi - 1) >> a->h.log2_S, st, &v, &n, true);
   if (rc) return rc;
-  cudaError_t e = launch_gather(v, a->h.log2_S, lo, hi, static_cast<uint8_t *>(d_out), st);
-  if (e == cudaSuccess) e = launch_clear_pages(a->d_page.p, a->d_work.p, n, st);
-  return cuda_status(e);
+  return cuda_status(launch_gather(v, a->h.log2_S, lo, hi, static_cast<uint8_t *>(d_out), a->d_page.p, a->d_work.p, n, st));
 }
 
 int aceapex_range_closure(aceapex_archive *a, uint64_t lo, uint64_t hi, uint64_t *n_segments, uint32_t *max_level) {
@@ -938,10 +943,8 @@ int aceapex_decode_region(aceapex_archive *a, uint64_t chrom, uint64_t pos, uint
   uint32_t n = 0;
   rc = decode_closure(a, lo >> a->h.log2_S, (hi - 1) >> a->h.log2_S, st, &v, &n, true);
   if (rc) return rc;
-  cudaError_t e = launch_gather_bases(v, a->h.log2_S, lo, (uint32_t)(pos % line_width), line_width, len,
-                                      static_cast<uint8_t *>(d_out), st);
-  if (e == cudaSuccess) e = launch_clear_pages(a->d_page.p, a->d_work.p, n, st);
-  return cuda_status(e);
+  return cuda_status(launch_gather_bases(v, a->h.log2_S, lo, (uint32_t)(pos % line_width), line_width, len,
+                                         static_cast<uint8_t *>(d_out), a->d_page.p, a->d_work.p, n, st));
 }
 
 int aceapex_last_error(aceapex_archive *a, int sync, void *stream) {

@@ -1501,6 +1501,22 @@ __global__ void init_flags_kernel(uint64_t *flags, const SegRec *dir, uint64_t n
   if (s < n) flags[s] = (uint64_t)dir[s].level << 32;
 }
 
+// A range decode's list by value: writes the work list and the page table and
+// starts the call, in one launch (a copy from pinned memory and two kernels
+// took 8 us before the decode could start).
+__global__ void __launch_bounds__(1024) begin_list_kernel(const __grid_constant__ WorkList list, WorkItem *work,
+                                                          uint32_t *page, uint32_t *global_epoch, uint32_t *epoch,
+                                                          uint32_t *counter) {
+  if (threadIdx.x == 0) {
+    *epoch = atomicAdd(global_epoch, 1u) + 1u;
+    *counter = 0;
+  }
+  if (threadIdx.x < list.n) {
+    work[threadIdx.x] = WorkItem{0u, list.seg[threadIdx.x]};
+    page[list.seg[threadIdx.x]] = threadIdx.x;
+  }
+}
+
 __global__ void begin_kernel(uint32_t *global_epoch, uint32_t *epoch, uint32_t *counter) {
   *epoch = atomicAdd(global_epoch, 1u) + 1u;
   *counter = 0;
@@ -1555,14 +1571,31 @@ __global__ void gather_kernel(OutView v, uint32_t log2_S, uint64_t lo, uint64_t 
   }
 }
 
+// gather_kernel for a short range, and the page table's entries cleared after
+// it, by one CTA
+__global__ void __launch_bounds__(1024) gather_clear_kernel(OutView v, uint32_t log2_S, uint64_t lo, uint64_t n,
+                                                            uint8_t *dst, uint32_t *page, const WorkItem *work,
+                                                            uint32_t n_work) {
+  const uint64_t off = reinterpret_cast<uintptr_t>(dst) & 15, blocks = (off + n + 15) >> 4;
+  for (uint64_t k = threadIdx.x; k < blocks; k += blockDim.x)
+    gather_block(v, log2_S, lo, dst, k ? 16 * k - off : 0, min(n, 16 * (k + 1) - off));
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < n_work; i += blockDim.x) page[work[i].seg] = 0xFFFFFFFFu;
+}
+
 // bases [0, n) of a FASTA region whose first base sits at lo with line phase
 // `phase` (its position within a line of L bases): base i is at
 // lo + i + (phase + i) / L, the newline after every L bases skipped
+// (with n_work, by one CTA, which then clears the page table's entries)
 __global__ void gather_bases_kernel(OutView v, uint32_t log2_S, uint64_t lo, uint32_t phase, uint32_t L, uint64_t n,
-                                    uint8_t *dst) {
+                                    uint8_t *dst, uint32_t *page, const WorkItem *work, uint32_t n_work) {
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
     const uint8_t *p = at(v, lo + i + (phase + i) / L, log2_S);
     dst[i] = p ? *p : 0;
+  }
+  if (n_work) {
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < n_work; i += blockDim.x) page[work[i].seg] = 0xFFFFFFFFu;
   }
 }
 
@@ -2088,6 +2121,12 @@ cudaError_t launch_init_flags(uint64_t *flags, const SegRec *dir, uint64_t n, cu
   return cudaGetLastError();
 }
 
+cudaError_t launch_begin_list(const WorkList &list, WorkItem *work, uint32_t *page, uint32_t *global_epoch,
+                              uint32_t *epoch, uint32_t *counter, cudaStream_t st) {
+  begin_list_kernel<<<1, 1024, 0, st>>>(list, work, page, global_epoch, epoch, counter);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_begin(uint32_t *global_epoch, uint32_t *epoch, uint32_t *counter, cudaStream_t st) {
   begin_kernel<<<1, 1, 0, st>>>(global_epoch, epoch, counter);
   return cudaGetLastError();
@@ -2107,20 +2146,32 @@ cudaError_t launch_copy_view(OutView src, OutView dst, uint32_t log2_S, uint64_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather(OutView v, uint32_t log2_S, uint64_t lo, uint64_t hi, uint8_t *dst, cudaStream_t st) {
-  if (hi <= lo) return cudaSuccess;
+// Ranges up to this many bytes are gathered by one CTA, which clears the page
+// table too (a lookup's record or region: one launch of 3 us instead of two).
+constexpr uint64_t kShortGather = 16384;
+
+cudaError_t launch_gather(OutView v, uint32_t log2_S, uint64_t lo, uint64_t hi, uint8_t *dst, uint32_t *page,
+                          const WorkItem *work, uint32_t n_work, cudaStream_t st) {
+  if (hi - lo <= kShortGather) {
+    gather_clear_kernel<<<1, 1024, 0, st>>>(v, log2_S, lo, hi - lo, dst, page, work, n_work);
+    return cudaGetLastError();
+  }
   const uint64_t n = hi - lo, want = (n / 16 + 2 + 255) / 256;  // (up to two partial blocks)
   const int grid = (int)(want < 4096 ? want : 4096);
   gather_kernel<<<grid, 256, 0, st>>>(v, log2_S, lo, n, dst);
-  return cudaGetLastError();
+  return launch_clear_pages(page, work, n_work, st);
 }
 
 cudaError_t launch_gather_bases(OutView v, uint32_t log2_S, uint64_t lo, uint32_t phase, uint32_t line_width,
-                                uint64_t n, uint8_t *dst, cudaStream_t st) {
-  if (!n) return cudaSuccess;
+                                uint64_t n, uint8_t *dst, uint32_t *page, const WorkItem *work, uint32_t n_work,
+                                cudaStream_t st) {
+  if (n <= kShortGather) {
+    gather_bases_kernel<<<1, 1024, 0, st>>>(v, log2_S, lo, phase, line_width, n, dst, page, work, n_work);
+    return cudaGetLastError();
+  }
   int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  gather_bases_kernel<<<grid, 256, 0, st>>>(v, log2_S, lo, phase, line_width, n, dst);
-  return cudaGetLastError();
+  gather_bases_kernel<<<grid, 256, 0, st>>>(v, log2_S, lo, phase, line_width, n, dst, nullptr, nullptr, 0);
+  return launch_clear_pages(page, work, n_work, st);
 }
 
 cudaError_t launch_fastq_interleave(const uint8_t *const base[4], const uint64_t len[4], uint32_t *counts,

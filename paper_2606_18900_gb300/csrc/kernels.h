@@ -79,6 +79,17 @@ struct LaunchShape {
 // fresh epochs.
 cudaError_t launch_begin(uint32_t *global_epoch, uint32_t *epoch, uint32_t *counter, cudaStream_t st);
 
+// A short list of segments passed to a kernel by value (with the kernel's
+// other arguments below the 4 KiB that launches take without a copy).
+constexpr uint32_t kListMax = 992;
+struct WorkList {
+  uint32_t n;
+  uint32_t seg[kListMax];
+};
+// work[i] = list.seg[i] and page[list.seg[i]] = i for i < list.n, and launch_begin
+cudaError_t launch_begin_list(const WorkList &list, WorkItem *work, uint32_t *page, uint32_t *global_epoch,
+                              uint32_t *epoch, uint32_t *counter, cudaStream_t st);
+
 // flags[s] = dir[s].level << 32 for s < n: each segment's flag word with its
 // level and no epoch
 cudaError_t launch_init_flags(uint64_t *flags, const SegRec *dir, uint64_t n, cudaStream_t st);
@@ -105,13 +116,16 @@ cudaError_t launch_batch(const DecodeLaunch &L, uint32_t n_arcs, int grid, cudaS
 // Occupancy-derived grid for the decode kernel.
 int decode_grid(int device, int block);
 
-// Gather [lo, hi) through a view into a flat buffer.
-cudaError_t launch_gather(OutView v, uint32_t log2_S, uint64_t lo, uint64_t hi, uint8_t *dst, cudaStream_t st);
+// Gather [lo, hi) through a paged view into a flat buffer, then clear the
+// page-table entries of work[0 .. n_work).
+cudaError_t launch_gather(OutView v, uint32_t log2_S, uint64_t lo, uint64_t hi, uint8_t *dst, uint32_t *page,
+                          const WorkItem *work, uint32_t n_work, cudaStream_t st);
 
 // n FASTA bases from lo (line phase `phase`, lines of line_width bases each
-// followed by a newline) into a flat buffer, newlines dropped
+// followed by a newline) into a flat buffer, newlines dropped, then the same
 cudaError_t launch_gather_bases(OutView v, uint32_t log2_S, uint64_t lo, uint32_t phase, uint32_t line_width,
-                                uint64_t n, uint8_t *dst, cudaStream_t st);
+                                uint64_t n, uint8_t *dst, uint32_t *page, const WorkItem *work, uint32_t n_work,
+                                cudaStream_t st);
 
 // page[work[i].seg] = i for i < n (paged views)
 cudaError_t launch_set_pages(uint32_t *page, const WorkItem *work, uint32_t n, cudaStream_t st);
