@@ -1137,6 +1137,7 @@ int aceapex_decode_batch(aceapex_archive *const *as, int n, void *const *d_outs,
   DecodeLaunch L = base_launch(A);
   L.arcs = A->d_batch_arcs.p;
   L.views = A->d_batch_views.p;
+  L.max_stage = need;  // of all archives
   return cuda_status(launch_batch(L, m, A->grid, st));
 }
 

@@ -1431,6 +1431,7 @@ __global__ void __launch_bounds__(kStagedThreads, 1) staged_kernel(DecodeLaunch 
 }
 
 // Batch decode, one archive per CTA at a time (see launch_batch).
+template <bool kSharedStage>
 __global__ void __launch_bounds__(kDecodeThreads, 1) batch_kernel(DecodeLaunch L, uint32_t n_arcs) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ uint32_t s_arc, s_next;
@@ -1466,7 +1467,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) batch_kernel(DecodeLaunch L
       if (idx >= A.n_seg) break;
       if (failed) continue;
       PHASE_MARK(5);
-      decode_segment<true, kViewLinear, false>(L, A, s_V, A.order[idx].seg, epoch, ws.lut, ws.stage, L.stage_cap,
+      decode_segment<true, kViewLinear, kSharedStage>(L, A, s_V, A.order[idx].seg, epoch, ws.lut, ws.stage, L.stage_cap,
                                                gstage, ws.mt, ws.ring, lane, ph, ph_t);
     }
     __syncthreads();  // the table is replaced only after every warp left this archive
@@ -2039,9 +2040,10 @@ int decode_grid(int device, int block) {
   for (const void *k : {(const void *)staged_kernel<kViewLinear>, (const void *)staged_kernel<kViewRing>,
                         (const void *)staged_kernel<kViewPaged>})
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem);
-  cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLutBytes);
+  smem((const void *)batch_kernel<false>);
+  smem((const void *)batch_kernel<true>);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_kernel<kViewLinear, false>, kDecodeThreads, kSmemLutBytes);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, batch_kernel, kDecodeThreads, kSmemLutBytes);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, batch_kernel<false>, kDecodeThreads, kSmemLutBytes);
   int per_sm = a < b ? a : b;
   if (per_sm < 1) per_sm = 1;
   return sms * per_sm;
@@ -2102,8 +2104,9 @@ cudaError_t launch_decode(const DecodeLaunch &L0, int grid, int block, cudaStrea
 
 cudaError_t launch_batch(const DecodeLaunch &L, uint32_t n_arcs, int grid, cudaStream_t st) {
   if (n_arcs == 0) return cudaSuccess;
-  cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLutBytes);
-  batch_kernel<<<grid, kDecodeThreads, kSmemLutBytes, st>>>(L, n_arcs);
+  // (as launch_decode: the stage-in-shared kernel when every segment of every archive fits)
+  if (L.max_stage <= L.stage_cap) batch_kernel<true><<<grid, kDecodeThreads, kSmemLutBytes, st>>>(L, n_arcs);
+  else batch_kernel<false><<<grid, kDecodeThreads, kSmemLutBytes, st>>>(L, n_arcs);
   return cudaGetLastError();
 }
 
