@@ -1138,7 +1138,9 @@ int aceapex_decode_batch(aceapex_archive *const *as, int n, void *const *d_outs,
   L.arcs = A->d_batch_arcs.p;
   L.views = A->d_batch_views.p;
   L.max_stage = need;  // of all archives
-  return cuda_status(launch_batch(L, m, A->grid, st));
+  uint32_t small = 0;
+  while (small < m && as[perm[m - 1 - small]]->h.n_seg <= kBatchSmall) ++small;
+  return cuda_status(launch_batch(L, m, small, A->grid, st));
 }
 
 int aceapex_encode(const void *h_in, uint64_t n, uint32_t log2_B, uint32_t min_match, uint32_t max_level,

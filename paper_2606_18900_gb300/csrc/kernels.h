@@ -110,8 +110,10 @@ cudaError_t launch_copy_view(OutView src, OutView dst, uint32_t log2_S, uint64_t
 
 // Batch decode: each CTA takes whole archives (L.arcs[0..n_arcs), largest
 // first) and decodes each archive's segments in its level order with the
-// archive's decode table in shared memory. L.work is unused.
-cudaError_t launch_batch(const DecodeLaunch &L, uint32_t n_arcs, int grid, cudaStream_t st);
+// archive's decode table in shared memory; the last n_small archives have at
+// most kBatchSmall segments each and may share a CTA. L.work is unused.
+constexpr uint32_t kBatchSmall = 9;
+cudaError_t launch_batch(const DecodeLaunch &L, uint32_t n_arcs, uint32_t n_small, int grid, cudaStream_t st);
 
 // Occupancy-derived grid for the decode kernel.
 int decode_grid(int device, int block);
