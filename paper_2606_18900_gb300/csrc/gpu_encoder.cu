@@ -451,13 +451,18 @@ __global__ void __launch_bounds__(256) rs_scatter_kernel(const uint32_t *kin, co
 // test there only saves comparing, so it has no counterpart here). A pair is
 // compared over kGoodEnough bytes at most: the first pair that long ends its
 // slot's walk, and only that one's full length is needed. 192 MiB of FASTQ:
-// 18.3 -> 13.3 ms.
+// 18.3 -> 12.9 ms.
 //
 // The length from kGoodEnough on of the match of p from c. (Out of line: few
 // slots come here; inlined it costs the kernel 0.4 ms in registers.)
 __device__ __noinline__ uint64_t long_match(const ParseCtx &g, uint64_t c, uint64_t p) {
   return kGoodEnough + common_len(g.in + c + kGoodEnough, g.in + p + kGoodEnough, match_limit(g, c, p) - kGoodEnough);
 }
+// Pairs of a warp (of at most 512) that are spread over its lanes. With more,
+// most slots have long chains: a thread per slot leaves few lanes waiting, and
+// the 8-byte test pays (16 MB of genome, min_match 32: 0.38 ms against 1.15
+// with every warp's pairs spread; 192 MiB of FASTQ 12.9 against 13.4).
+constexpr uint32_t kPairsMost = 256;
 constexpr uint32_t kMatchStop = 0xffffffffu;  // this candidate and the later ones are too far away
 constexpr uint32_t kMatchFull = 0x80000000u;  // the match reaches the end of the segment
 __global__ void __launch_bounds__(256) enc_match_kernel(ParseCtx g, const uint32_t *K, const uint32_t *V, uint64_t m,
@@ -496,6 +501,14 @@ __global__ void __launch_bounds__(256) enc_match_kernel(ParseCtx g, const uint32
       if (lane >= (uint32_t)o) incl += y;
     }
     const uint32_t first = incl - n, total = __shfl_sync(kFull, incl, 31);
+    if (total > kPairsMost) {
+      if (n) {
+        uint64_t src;
+        const uint64_t L = match_at_slot(g, K, V, j, p, &src);
+        if (L) table[p - a] = L << 32 | (p - src);
+      }
+      continue;
+    }
     for (uint32_t t0 = 0; t0 < total; t0 += 32) {
       const uint32_t t = t0 + lane;
       uint32_t s = 0;  // the slot of pair t: the last one whose pairs start at or before t

@@ -21,6 +21,9 @@
 //      stores before what lane 0 does next), then lane 0 stores the level and
 //      epoch into the segment's flag with release semantics, a release that
 //      covers the other lanes' stores through that ordering.
+// staged_kernel — the same for short lists, where latency counts: a team of
+// warps per segment, built in shared memory.
+// batch_kernel — whole archives per CTA, or two small ones.
 // Errors latch the first code into a device word; waits give up at a time
 // limit (globaltimer) or as soon as another warp has latched an error.
 #include <cuda_runtime.h>
