@@ -670,7 +670,7 @@ def workload_fastq_streams(args):
                       "ratio_gain_pct": round(100 * (single.size / comp - 1), 1),
                       "split_seconds": round(split_s, 2), "encode_seconds": round(enc_s, 2),
                       "l2": "inputs larger than L2"},
-                     gpu_launches=args.steps * (2 * 4 + 3 * 4 + 1), bit_exact=ok, ms_median=float(np.median(step_ms)))
+                     gpu_launches=args.steps * (2 * 4 + 4), bit_exact=ok, ms_median=float(np.median(step_ms)))
     print(json.dumps(line), flush=True)
     for p_ in parts:
         p_.close()
@@ -981,7 +981,7 @@ def workload_genome(args):
                      coordinate_region={"p50_ms": pctl(coord_lat, 50), "p99_ms": pctl(coord_lat, 99),
                                         "n": len(coord_lat), "bit_exact": bool(coord_ok),
                                         "what": "150 bases at (record, position), aceapex_decode_region, synchronous"},
-                     batched_regions=batched, crc_windows_match=ok, gpu_launches=args.steps * (1 + 3 * nw),
+                     batched_regions=batched, crc_windows_match=ok, gpu_launches=args.steps * (1 + 2 * nw),
                      bit_exact=bool(ok and reg_ok and coord_ok and b_ok))
     print(json.dumps(line), flush=True)
 
