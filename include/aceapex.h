@@ -382,8 +382,8 @@ uint64_t aceapex_fastq_split(const void *h_in, uint64_t n, void *h_out, uint64_t
 /*
  * Whole-file decode of a FASTQ stored as four archives of its line streams
  * (parts[k] holds stream k of aceapex_fastq_split): each part decodes with
- * its own persistent launch into scratch owned by parts[0], a newline index
- * of each stream is built on the device, and one warp per record copies its
+ * its own persistent launch, side by side, into scratch owned by parts[0], a newline index
+ * of each stream is built on the device, and each record is copied from its
  * four lines to d_out[0 .. N), N the sum of the streams' sizes. Stream-
  * ordered; decode errors are latched in each part's error word, and a
  * stream that is not made of FASTQ lines in parts[0]'s. Each stream must be below 4 GiB. Errors:
