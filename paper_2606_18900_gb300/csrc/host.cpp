@@ -435,7 +435,7 @@ int device_closure(aceapex_archive *A, uint64_t s_lo, uint64_t s_hi, cudaStream_
   if (!A->d_dep_ptr.p) {
     if (A->d_dep_ptr.alloc(ns + 1) != cudaSuccess || A->d_deps.alloc(std::max<uint64_t>(A->h.n_deps, 1)) != cudaSuccess ||
         A->d_cmark.alloc(ns) != cudaSuccess || A->d_clist.alloc(ns) != cudaSuccess ||
-        A->d_ccnt.alloc(4) != cudaSuccess || A->stage_cnt.reserve(16) != cudaSuccess)
+        A->d_ccnt.alloc(kClosureFound + 1) != cudaSuccess || A->stage_cnt.reserve(16) != cudaSuccess)
       return ACEAPEX_ENOMEM;
     if (cudaMemcpy(A->d_dep_ptr.p, A->dep_ptr.data(), 8 * (ns + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
         (A->h.n_deps &&
@@ -453,13 +453,15 @@ int device_closure(aceapex_archive *A, uint64_t s_lo, uint64_t s_hi, cudaStream_
     if (cudaMemsetAsync(A->d_cmark.p, 0, 4 * ns, st) != cudaSuccess) return ACEAPEX_ECUDA;
     A->cgen = 1;
   }
-  ClosureDev C{A->d_dep_ptr.p, A->d_deps.p, A->d_dir.p, A->d_cmark.p, A->d_clist.p, A->d_ccnt.p};
+  ClosureDev C{A->d_dep_ptr.p, A->d_deps.p, A->d_dir.p, A->d_cmark.p, A->d_clist.p, A->d_ccnt.p, A->err(),
+               (uint32_t)ns};
+  uint32_t *const n_dev = A->d_ccnt.p + kClosureFound;
   uint32_t top = 0;
   for (uint64_t s = s_lo; s <= s_hi; ++s) top = std::max<uint32_t>(top, A->dir[s].level);
-  cudaError_t e = launch_closure_seed(C, (uint32_t)s_lo, (uint32_t)(s_hi - s_lo + 1), A->cgen, st);
-  for (uint32_t l = top; e == cudaSuccess && l >= 1; --l) e = launch_closure_expand(C, l, A->cgen, st);
-  if (e == cudaSuccess) e = launch_closure_order(C, A->d_work.p, A->d_page.p, A->d_ccnt.p + 1, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(A->stage_cnt.p, A->d_ccnt.p + 1, 4, cudaMemcpyDeviceToHost, st);
+  cudaError_t e = launch_closure_seed(C, (uint32_t)s_lo, (uint32_t)(s_hi - s_lo + 1), top, A->cgen, st);
+  for (uint32_t l = top; e == cudaSuccess && l >= 1; --l) e = launch_closure_expand(C, l, top, A->cgen, st);
+  if (e == cudaSuccess) e = launch_closure_order(C, top, A->d_work.p, A->d_page.p, n_dev, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(A->stage_cnt.p, n_dev, 4, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return ACEAPEX_ECUDA;
   *n_out = *static_cast<const uint32_t *>(A->stage_cnt.p);

@@ -1663,26 +1663,42 @@ __global__ void set_pages_kernel(uint32_t *page, const WorkItem *work, uint32_t 
 }
 
 // -------------------------------------------------------- device closures
-__global__ void closure_seed_kernel(ClosureDev C, uint32_t s_lo, uint32_t n, uint32_t gen) {
+// Members are only read from list slots that an earlier launch has filled:
+// found[l] counts what expanding level l added, found[top + 1] the seeds, so
+// the members before level l's launch are the sum over the levels above l, all
+// of them words that no warp of that launch writes. (One counter for all
+// levels would rise while its launch still runs, and before the slots behind
+// it are written.)
+__device__ __forceinline__ uint32_t closure_settled(const ClosureDev &C, uint32_t level, uint32_t top, int lane) {
+  uint32_t n = 0;
+  for (uint32_t l = level + 1 + lane; l <= top + 1; l += 32) n += C.found[l];
+  return __reduce_add_sync(kFull, n);
+}
+
+__global__ void closure_seed_kernel(ClosureDev C, uint32_t s_lo, uint32_t n, uint32_t top, uint32_t gen) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     C.mark[s_lo + i] = gen;
     C.list[i] = s_lo + i;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *C.cnt = n;
+  if (blockIdx.x == 0)
+    for (uint32_t l = threadIdx.x; l <= top + 1; l += blockDim.x) C.found[l] = l == top + 1 ? n : 0u;
 }
 
 // One warp per member of the given level (grid-stride over the list); its
 // lanes walk the member's dependency list. A dependency joins the closure
 // when this warp is the first to tag it with gen; the warp reserves the list
 // slots of its new members with one atomic. Members added here have lower
-// levels, so the entries a warp sees beyond its first reading of cnt are
-// skipped by the level test.
-__global__ void closure_expand_kernel(ClosureDev C, uint32_t level, uint32_t gen) {
+// levels, so the list that this level needs is complete before its launch.
+__global__ void closure_expand_kernel(ClosureDev C, uint32_t level, uint32_t top, uint32_t gen) {
   const int lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-  const uint32_t n = ld_relaxed(C.cnt);
+  const uint32_t n = closure_settled(C, level, top, lane);
   for (uint32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
     const uint32_t s = C.list[i];
+    if (s >= C.n_seg) {  // (a slot that nobody wrote: nothing is read through it)
+      if (lane == 0) latch(C.err, kErrCorrupt);
+      continue;
+    }
     if (C.dir[s].level != level) continue;
     const uint64_t b = C.dep_ptr[s], e = C.dep_ptr[s + 1];
     for (uint64_t k0 = b; k0 < e; k0 += 32) {
@@ -1696,37 +1712,41 @@ __global__ void closure_expand_kernel(ClosureDev C, uint32_t level, uint32_t gen
       const uint32_t m = __ballot_sync(kFull, fresh);
       if (!m) continue;
       uint32_t base = 0;
-      if (lane == 0) base = atomicAdd(C.cnt, (uint32_t)__popc(m));
+      if (lane == 0) base = n + atomicAdd(C.found + level, (uint32_t)__popc(m));
       base = __shfl_sync(kFull, base, 0);
       if (fresh) C.list[base + __popc(m & lanemask_lt())] = d;
     }
   }
 }
 
-// one CTA: counting sort of the members by level (levels < 65536)
-constexpr int kClosureLevels = 256;
-__global__ void __launch_bounds__(1024) closure_order_kernel(ClosureDev C, WorkItem *work, uint32_t *page,
-                                                             uint32_t *n_out) {
+// one CTA: counting sort of the members by level (a level is one byte)
+__global__ void __launch_bounds__(1024) closure_order_kernel(ClosureDev C, uint32_t top, WorkItem *work,
+                                                             uint32_t *page, uint32_t *n_out) {
   __shared__ uint32_t off[kClosureLevels];
-  const uint32_t n = *C.cnt;
-  for (int l = threadIdx.x; l < kClosureLevels; l += blockDim.x) off[l] = 0;
+  const uint32_t n = closure_settled(C, 0, top, threadIdx.x & 31);
+  for (uint32_t l = threadIdx.x; l < kClosureLevels; l += blockDim.x) off[l] = 0;
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x)
-    atomicAdd(&off[min((uint32_t)C.dir[C.list[i]].level, (uint32_t)(kClosureLevels - 1))], 1u);
+  auto level_of = [&](uint32_t s) { return min((uint32_t)C.dir[s].level, kClosureLevels - 1); };
+  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+    const uint32_t s = C.list[i];
+    if (s < C.n_seg) atomicAdd(&off[level_of(s)], 1u);
+    else latch(C.err, kErrCorrupt);
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     uint32_t run = 0;
-    for (int l = 0; l < kClosureLevels; ++l) {
+    for (uint32_t l = 0; l < kClosureLevels; ++l) {
       const uint32_t c = off[l];
       off[l] = run;
       run += c;
     }
-    *n_out = n;
+    *n_out = run;
   }
   __syncthreads();
   for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
     const uint32_t s = C.list[i];
-    const uint32_t pos = atomicAdd(&off[min((uint32_t)C.dir[s].level, (uint32_t)(kClosureLevels - 1))], 1u);
+    if (s >= C.n_seg) continue;
+    const uint32_t pos = atomicAdd(&off[level_of(s)], 1u);
     work[pos] = WorkItem{0u, s};
     page[s] = pos;
   }
@@ -2257,21 +2277,22 @@ cudaError_t launch_set_pages(uint32_t *page, const WorkItem *work, uint32_t n, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_closure_seed(ClosureDev C, uint32_t s_lo, uint32_t n, uint32_t gen, cudaStream_t st) {
-  closure_seed_kernel<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, st>>>(C, s_lo, n, gen);
+cudaError_t launch_closure_seed(ClosureDev C, uint32_t s_lo, uint32_t n, uint32_t top, uint32_t gen, cudaStream_t st) {
+  closure_seed_kernel<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, st>>>(C, s_lo, n, top, gen);
   return cudaGetLastError();
 }
 
-cudaError_t launch_closure_expand(ClosureDev C, uint32_t level, uint32_t gen, cudaStream_t st) {
+cudaError_t launch_closure_expand(ClosureDev C, uint32_t level, uint32_t top, uint32_t gen, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  closure_expand_kernel<<<2 * sms, 512, 0, st>>>(C, level, gen);
+  closure_expand_kernel<<<2 * sms, 512, 0, st>>>(C, level, top, gen);
   return cudaGetLastError();
 }
 
-cudaError_t launch_closure_order(ClosureDev C, WorkItem *work, uint32_t *page, uint32_t *n_out, cudaStream_t st) {
-  closure_order_kernel<<<1, 1024, 0, st>>>(C, work, page, n_out);
+cudaError_t launch_closure_order(ClosureDev C, uint32_t top, WorkItem *work, uint32_t *page, uint32_t *n_out,
+                                 cudaStream_t st) {
+  closure_order_kernel<<<1, 1024, 0, st>>>(C, top, work, page, n_out);
   return cudaGetLastError();
 }
 

@@ -156,24 +156,31 @@ cudaError_t launch_fastq_interleave(const uint8_t *const base[4], const uint64_t
 // Transitive source closure on the device, for range decodes whose closure
 // is too wide to walk on the host (paper §4.1: a read decodes its covering
 // blocks plus their sources). mark: one u32 per segment, equal to gen when the
-// segment is in the current closure; list: the members in discovery order;
-// cnt[0]: their number. Every dependency has a lower level than its reader, so
-// expanding the members of level L (max level down to 1) after all higher
-// levels visits each member once.
+// segment is in the current closure; list: the members in discovery order.
+// Every dependency has a lower level than its reader, so expanding the members
+// of level L (the seeds' highest level, top, down to 1, a launch each) after
+// all higher levels visits each member once. found: kClosureFound words,
+// found[top + 1] the number of seeds, found[L] the members that level L's
+// launch added. A member that is no segment latches an error in *err.
+constexpr uint32_t kClosureLevels = 256;  // a level is one byte in the archive's header
+constexpr uint32_t kClosureFound = kClosureLevels + 1;
 struct ClosureDev {
   const uint64_t *dep_ptr;
   const uint32_t *deps;
   const SegRec *dir;
   uint32_t *mark;
   uint32_t *list;
-  uint32_t *cnt;
+  uint32_t *found;
+  uint32_t *err;
+  uint32_t n_seg;
 };
 // members := segments [s_lo, s_lo + n)
-cudaError_t launch_closure_seed(ClosureDev C, uint32_t s_lo, uint32_t n, uint32_t gen, cudaStream_t st);
+cudaError_t launch_closure_seed(ClosureDev C, uint32_t s_lo, uint32_t n, uint32_t top, uint32_t gen, cudaStream_t st);
 // add the unmarked dependencies of every member of level `level`
-cudaError_t launch_closure_expand(ClosureDev C, uint32_t level, uint32_t gen, cudaStream_t st);
+cudaError_t launch_closure_expand(ClosureDev C, uint32_t level, uint32_t top, uint32_t gen, cudaStream_t st);
 // members sorted by level into work[0 .. n), page[seg] = its position, n into *n_out
-cudaError_t launch_closure_order(ClosureDev C, WorkItem *work, uint32_t *page, uint32_t *n_out, cudaStream_t st);
+cudaError_t launch_closure_order(ClosureDev C, uint32_t top, WorkItem *work, uint32_t *page, uint32_t *n_out,
+                                 cudaStream_t st);
 
 // CRC-32 of [lo, hi) of the ring view, written to *crc; sums: two device words
 // that are zero between launches.
