@@ -68,13 +68,17 @@ struct Staging {
   bool pending = false;
   cudaError_t reserve(uint64_t b) {
     if (pending) cudaEventSynchronize(done), pending = false;
+    if (!done) {
+      const cudaError_t e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+      if (e != cudaSuccess) return done = nullptr, e;
+    }
     if (b <= bytes) return cudaSuccess;
     if (p) cudaFreeHost(p);
     p = nullptr;
     bytes = 0;
-    cudaError_t e = cudaMallocHost(&p, b);
+    const cudaError_t e = cudaMallocHost(&p, b);
     if (e == cudaSuccess) bytes = b;
-    if (!done) cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+    else p = nullptr;
     return e;
   }
   void mark(cudaStream_t st) {

@@ -40,8 +40,13 @@ uint32_t *global_epoch(int device) {
   std::lock_guard<std::mutex> lk(g_dev_mu);
   DeviceState &d = g_dev[device];
   if (!d.d_global_epoch) {
-    if (cudaMalloc(&d.d_global_epoch, sizeof(uint32_t)) != cudaSuccess) return nullptr;
-    if (cudaMemset(d.d_global_epoch, 0, sizeof(uint32_t)) != cudaSuccess) return nullptr;
+    uint32_t *p = nullptr;
+    if (cudaMalloc(&p, sizeof(uint32_t)) != cudaSuccess) return nullptr;
+    if (cudaMemset(p, 0, sizeof(uint32_t)) != cudaSuccess) {
+      cudaFree(p);
+      return nullptr;
+    }
+    d.d_global_epoch = p;
   }
   return d.d_global_epoch;
 }
@@ -432,17 +437,19 @@ constexpr uint64_t kHostClosureEdges = 16384;
 // stream synchronisation) so that the arena can be sized for it.
 int device_closure(aceapex_archive *A, uint64_t s_lo, uint64_t s_hi, cudaStream_t st, uint32_t *n_out) {
   const uint64_t ns = A->h.n_seg;
-  if (!A->d_dep_ptr.p) {
-    if (A->d_dep_ptr.alloc(ns + 1) != cudaSuccess || A->d_deps.alloc(std::max<uint64_t>(A->h.n_deps, 1)) != cudaSuccess ||
-        A->d_cmark.alloc(ns) != cudaSuccess || A->d_clist.alloc(ns) != cudaSuccess ||
-        A->d_ccnt.alloc(kClosureFound + 1) != cudaSuccess || A->stage_cnt.reserve(16) != cudaSuccess)
+  if (!A->d_dep_ptr.p) {  // (allocated last and given up if the set-up fails: its presence says that all is there)
+    if (A->d_deps.alloc(std::max<uint64_t>(A->h.n_deps, 1)) != cudaSuccess || A->d_cmark.alloc(ns) != cudaSuccess ||
+        A->d_clist.alloc(ns) != cudaSuccess || A->d_ccnt.alloc(kClosureFound + 1) != cudaSuccess ||
+        A->stage_cnt.reserve(16) != cudaSuccess || A->d_dep_ptr.alloc(ns + 1) != cudaSuccess)
       return ACEAPEX_ENOMEM;
     if (cudaMemcpy(A->d_dep_ptr.p, A->dep_ptr.data(), 8 * (ns + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
         (A->h.n_deps &&
          cudaMemcpy(A->d_deps.p, A->deps.data(), 4 * A->h.n_deps, cudaMemcpyHostToDevice) != cudaSuccess) ||
         cudaMemset(A->d_cmark.p, 0, 4 * ns) != cudaSuccess ||
-        cudaStreamSynchronize(0) != cudaSuccess)  // (st need not wait for the legacy stream)
+        cudaStreamSynchronize(0) != cudaSuccess) {  // (st need not wait for the legacy stream)
+      A->d_dep_ptr.release();
       return ACEAPEX_ECUDA;
+    }
     A->cgen = 0;
   }
   if (A->d_work.n < ns) {
@@ -450,7 +457,10 @@ int device_closure(aceapex_archive *A, uint64_t s_lo, uint64_t s_hi, cudaStream_
     if (A->d_work.alloc(ns) != cudaSuccess) return ACEAPEX_ENOMEM;
   }
   if (++A->cgen == 0) {  // tags wrapped: clear the marks
-    if (cudaMemsetAsync(A->d_cmark.p, 0, 4 * ns, st) != cudaSuccess) return ACEAPEX_ECUDA;
+    if (cudaMemsetAsync(A->d_cmark.p, 0, 4 * ns, st) != cudaSuccess) {
+      --A->cgen;  // (the next call clears them)
+      return ACEAPEX_ECUDA;
+    }
     A->cgen = 1;
   }
   ClosureDev C{A->d_dep_ptr.p, A->d_deps.p, A->d_dir.p, A->d_cmark.p, A->d_clist.p, A->d_ccnt.p, A->err(),
@@ -474,7 +484,10 @@ int decode_closure(aceapex_archive *A, uint64_t s_lo, uint64_t s_hi, cudaStream_
   const uint64_t S = uint64_t(1) << A->h.log2_S;
   if (!A->d_page.p) {
     if (A->d_page.alloc(A->h.n_seg) != cudaSuccess) return ACEAPEX_ENOMEM;
-    if (cudaMemsetAsync(A->d_page.p, 0xFF, 4 * A->h.n_seg, st) != cudaSuccess) return ACEAPEX_ECUDA;
+    if (cudaMemsetAsync(A->d_page.p, 0xFF, 4 * A->h.n_seg, st) != cudaSuccess) {
+      A->d_page.release();  // (a table that was not filled is not kept)
+      return ACEAPEX_ECUDA;
+    }
   }
   std::vector<uint32_t> segs;
   if (!closure(A, s_lo, s_hi, segs, kHostClosureEdges)) {
@@ -697,6 +710,7 @@ int prepare_windows(aceapex_archive *a, uint64_t window, cudaStream_t st) {
     // window k is segments [k per, (k + 1) per), and its work list sits at
     // the same place of the window lists, made on the device
     const uint64_t per = window / S;
+    a->win_bytes = 0;  // (no size until all of it is made)
     a->win_start.clear();
     for (uint64_t s = 0; s < a->h.n_seg; s += per) a->win_start.push_back(s);
     a->win_start.push_back(a->h.n_seg);
@@ -1024,7 +1038,10 @@ int aceapex_stream_range(aceapex_archive *a, uint64_t lo, uint64_t hi, uint64_t 
   }
   if (!a->d_crc_sums.p) {
     if (a->d_crc_sums.alloc(2) != cudaSuccess) return ACEAPEX_ENOMEM;
-    if (cudaMemsetAsync(a->d_crc_sums.p, 0, 8, st) != cudaSuccess) return ACEAPEX_ECUDA;
+    if (cudaMemsetAsync(a->d_crc_sums.p, 0, 8, st) != cudaSuccess) {
+      a->d_crc_sums.release();
+      return ACEAPEX_ECUDA;
+    }
   }
   OutView ring{};
   ring.base = a->d_ring.p;
@@ -1119,7 +1136,8 @@ int aceapex_decode_batch(aceapex_archive *const *as, int n, void *const *d_outs,
   std::memcpy(desc.data(), arcs.data(), sizeof(DevArchive) * m);
   std::memcpy(desc.data() + sizeof(DevArchive) * m, views.data(), sizeof(OutView) * m);
   if (desc != A->batch_desc) {
-    if (A->d_batch_arcs.n < m) {
+    A->batch_desc.clear();  // (the device's copy is no call's description until both parts are copied)
+    if (A->d_batch_arcs.n < m || A->d_batch_views.n < m) {
       cudaStreamSynchronize(st);
       if (A->d_batch_arcs.alloc(m) != cudaSuccess || A->d_batch_views.alloc(m) != cudaSuccess) return ACEAPEX_ENOMEM;
     }
@@ -1219,9 +1237,8 @@ int aceapex_decode_fastq_streams(aceapex_archive *const *parts, void *d_out, uin
   int rc = ensure_scratch(A);
   if (rc) return rc;
   for (int k = 1; apart && k < 4; ++k)
-    if (!A->fq_st[k - 1] &&
-        (cudaStreamCreateWithFlags(&A->fq_st[k - 1], cudaStreamNonBlocking) != cudaSuccess ||
-         cudaEventCreateWithFlags(&A->fq_ev[k], cudaEventDisableTiming) != cudaSuccess))
+    if ((!A->fq_st[k - 1] && cudaStreamCreateWithFlags(&A->fq_st[k - 1], cudaStreamNonBlocking) != cudaSuccess) ||
+        (!A->fq_ev[k] && cudaEventCreateWithFlags(&A->fq_ev[k], cudaEventDisableTiming) != cudaSuccess))
       return ACEAPEX_ECUDA;
   if (apart && !A->fq_ev[0] && cudaEventCreateWithFlags(&A->fq_ev[0], cudaEventDisableTiming) != cudaSuccess)
     return ACEAPEX_ECUDA;

@@ -1,0 +1,40 @@
+"""The library's host code over a CUDA runtime that runs on the CPU
+(tests/support/host_on_fake_cuda.cpp): each entry point is called with each of
+its runtime calls failing in turn and then called again, which has to work and
+to launch nothing on memory that is missing, too small or not initialised."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+import synth
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    cuda = "/usr/local/cuda/include"
+    if not shutil.which("g++") or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
+        pytest.skip("no g++ or no CUDA headers")
+    csrc = os.path.join(ROOT, "paper_2606_18900_gb300", "csrc")
+    d = tmp_path_factory.mktemp("fake_cuda")
+    sources = [os.path.join(ROOT, "tests", "support", "host_on_fake_cuda.cpp")]
+    sources += [os.path.join(csrc, f) for f in ("host.cpp", "encoder.cpp")]
+    r = subprocess.run(["g++", "-std=c++17", "-O1", "-I" + csrc, "-I" + os.path.join(ROOT, "include"), "-I" + cuda,
+                        *sources, "-o", str(d / "program"), "-lpthread"], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    synth.pe_fastq(16 << 20, seed=12, ref_len=2_000_000).tofile(d / "in.fastq")
+
+    def run(mode):
+        r = subprocess.run([str(d / "program"), mode, str(d / "in.fastq")], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+        return r.stdout
+
+    return run
+
+
+def test_calls_after_a_failure(program):
+    out = program("calls")
+    assert out.count("ok ") == 9
