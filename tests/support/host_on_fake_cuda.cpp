@@ -1,5 +1,5 @@
 // Test helper (built by tests/test_host_on_fake_cuda.py): the library's host
-// code (host.cpp, encoder.cpp) over a CUDA runtime and kernel
+// code (host.cpp, server.cpp, encoder.cpp) over a CUDA runtime and kernel
 // launchers that run on the CPU. Device memory is heap memory filled with
 // 0xAB, which nothing may take for initialised; every runtime call and every
 // launch can be made to fail; every launch checks that the memory it is given
@@ -7,14 +7,18 @@
 //
 // usage: host_on_fake_cuda calls <FASTQ file>   each entry point, with each of
 //          its runtime calls failing in turn, and then called again
+//        host_on_fake_cuda server <FASTQ file>  requests go on while the serving
+//          engine reads a batch's error word back
 // prints "ok" lines and exits 1 at the first violation.
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <chrono>
 #include <cstdio>
 #include <cstdlib>
 #include <fstream>
 #include <functional>
+#include <future>
 #include <iterator>
 #include <map>
 #include <mutex>
@@ -67,6 +71,8 @@ cudaError_t take(void *p) {
   return cudaSuccess;
 }
 
+std::function<void()> g_on_read_back;  // called inside every copy to the host
+
 }  // namespace
 
 extern "C" {
@@ -85,6 +91,7 @@ cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind k) {
   if (cudaError_t e = call()) return e;
   if (k != cudaMemcpyDeviceToHost) REQUIRE(live(d, n));
   if (k != cudaMemcpyHostToDevice) REQUIRE(live(s, n));
+  if (k == cudaMemcpyDeviceToHost && g_on_read_back) g_on_read_back();
   return std::memcpy(d, s, n), cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind k, cudaStream_t) {
@@ -210,6 +217,12 @@ cudaError_t launch_gather_bases(OutView, uint32_t, uint64_t, uint32_t, uint32_t,
 cudaError_t launch_copy_view(OutView a, OutView b, uint32_t, uint64_t, uint64_t, cudaStream_t) {
   REQUIRE(live(a.slot_base, 1) && live(b.base, b.mask + 1));
   return call();
+}
+cudaError_t launch_multi_gather(const GatherJob *jobs, uint32_t n, uint64_t, cudaStream_t) {
+  if (cudaError_t r = call()) return r;
+  REQUIRE(live(jobs, n * sizeof(GatherJob)));
+  for (uint32_t i = 0; i < n; ++i) REQUIRE(live(jobs[i].dst, jobs[i].n));
+  return cudaSuccess;
 }
 cudaError_t launch_fastq_interleave(const uint8_t *const base[4], const uint64_t len[4], uint32_t *counts,
                                     uint64_t *offs, uint32_t *const nl[4], const uint64_t cap[4], uint32_t *err,
@@ -368,6 +381,40 @@ void calls(const std::vector<uint8_t> &in) {
   REQUIRE(g_mem.size() <= 1);  // (the device's epoch word stays)
 }
 
+// Submits `n` ranges of the archive to a server and waits for them; returns
+// how many ended with a status other than OK.
+int serve(aceapex_server *S, int n, void *out) {
+  std::vector<uint64_t> tickets(n);
+  int bad = 0;
+  for (int i = 0; i < n; ++i)
+    REQUIRE(aceapex_server_submit(S, 0, 100 * i, 100 * i + 1000, out, 1000, &tickets[i]) == ACEAPEX_OK);
+  for (uint64_t t : tickets) {
+    int done = 0;
+    bad += aceapex_server_poll(S, t, 1, &done, nullptr) != ACEAPEX_OK;
+    REQUIRE(done);
+  }
+  return bad;
+}
+
+void server(const std::vector<uint8_t> &in) {
+  const auto arc = encoded(in.data(), 300'000, 14);
+  Opened o({&arc});
+  void *out = nullptr;
+  REQUIRE(cudaMalloc(&out, 1000) == cudaSuccess);
+  aceapex_server *S = nullptr;
+  REQUIRE(aceapex_server_create(o.as.data(), 1, 64 << 20, 4, &S) == ACEAPEX_OK);
+  g_on_read_back = [&] {
+    aceapex_server_stats st;
+    auto other = std::async(std::launch::async, [&] { return aceapex_server_get_stats(S, &st); });
+    REQUIRE(other.wait_for(std::chrono::seconds(10)) == std::future_status::ready);
+  };
+  REQUIRE(serve(S, 50, out) == 0);
+  aceapex_server_destroy(S);
+  g_on_read_back = nullptr;
+  take(out);
+  std::printf("ok requests go on while an error word is read back\n");
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -375,5 +422,6 @@ int main(int argc, char **argv) {
   std::ifstream f(argv[2], std::ios::binary);
   std::vector<uint8_t> in((std::istreambuf_iterator<char>(f)), std::istreambuf_iterator<char>());
   if (std::string(argv[1]) == "calls") calls(in);
+  else server(in);
   return 0;
 }

@@ -21,7 +21,7 @@ def program(tmp_path_factory):
     csrc = os.path.join(ROOT, "paper_2606_18900_gb300", "csrc")
     d = tmp_path_factory.mktemp("fake_cuda")
     sources = [os.path.join(ROOT, "tests", "support", "host_on_fake_cuda.cpp")]
-    sources += [os.path.join(csrc, f) for f in ("host.cpp", "encoder.cpp")]
+    sources += [os.path.join(csrc, f) for f in ("host.cpp", "server.cpp", "encoder.cpp")]
     r = subprocess.run(["g++", "-std=c++17", "-O1", "-I" + csrc, "-I" + os.path.join(ROOT, "include"), "-I" + cuda,
                         *sources, "-o", str(d / "program"), "-lpthread"], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
@@ -38,3 +38,8 @@ def program(tmp_path_factory):
 def test_calls_after_a_failure(program):
     out = program("calls")
     assert out.count("ok ") == 9
+
+
+def test_server_does_not_block_requests(program):
+    """The engine's lock is free while it reads a batch's error word back."""
+    assert "ok requests" in program("server")
