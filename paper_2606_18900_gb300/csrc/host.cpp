@@ -349,6 +349,11 @@ DecodeLaunch base_launch(aceapex_archive *A) {
   L.active_warps = A->active_warps;
   L.stage_cap = A->stage_cap;
   L.max_stage = A->max_cmd_syms;
+  // (team_shape says why) commands of a segment times levels against rANS
+  // steps of a segment, 32 symbols each: at least 1.4
+  const aceapex_stats &t = A->stats;
+  const uint64_t symbols = t.literal_bytes + t.n_commands * (4 + t.W);
+  L.team_rounds = 160 * t.n_commands * t.max_level >= 7 * symbols ? 2 : 1;
   return L;
 }
 

@@ -9,6 +9,8 @@
 //          its runtime calls failing in turn, and then called again
 //        host_on_fake_cuda server <FASTQ file>  requests go on while the serving
 //          engine reads a batch's error word back
+//        host_on_fake_cuda rounds <file>  prints how many segments one after
+//          the other its whole-file decode allows a team
 // prints "ok" lines and exits 1 at the first violation.
 #include <cuda_runtime.h>
 
@@ -130,6 +132,7 @@ cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t) { return cudaErrorNotSuppor
 namespace aceapex {
 
 int decode_grid(int, int) { return 152; }
+static uint32_t g_rounds;
 
 static bool archive_ok(const DevArchive &A) {
   return live(A.dir, 24 * (size_t)A.n_seg) && live(A.lut, kLutBytes) && live(A.flags, 8 * (size_t)A.n_seg) &&
@@ -184,6 +187,7 @@ cudaError_t launch_decode(const DecodeLaunch &L, int grid, int, cudaStream_t) {
   if (cudaError_t r = call()) return r;
   REQUIRE(grid > 0 && archive_ok(L.arc0) && live(L.work, 8 * (size_t)L.n_work));
   REQUIRE(live(L.err, 4) && live(L.epoch, 4) && live(L.counter, 4));
+  g_rounds = L.team_rounds;
   REQUIRE(L.max_stage <= L.stage_cap || live(L.scratch, (size_t)L.scratch_warps * kStageBytes));
   for (uint32_t i = 0; i < L.n_work; ++i) {
     REQUIRE(L.work[i].seg < L.arc0.n_seg);
@@ -415,6 +419,15 @@ void server(const std::vector<uint8_t> &in) {
   std::printf("ok requests go on while an error word is read back\n");
 }
 
+void rounds(const std::vector<uint8_t> &in) {
+  const auto arc = encoded(in.data(), in.size(), 14);
+  Opened o({&arc});
+  void *out = nullptr;
+  REQUIRE(cudaMalloc(&out, in.size()) == cudaSuccess);
+  REQUIRE(aceapex_decode_all(o.as[0], out, in.size(), nullptr, nullptr) == ACEAPEX_OK);
+  std::printf("rounds %u\n", g_rounds);
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -422,6 +435,7 @@ int main(int argc, char **argv) {
   std::ifstream f(argv[2], std::ios::binary);
   std::vector<uint8_t> in((std::istreambuf_iterator<char>(f)), std::istreambuf_iterator<char>());
   if (std::string(argv[1]) == "calls") calls(in);
-  else server(in);
+  else if (std::string(argv[1]) == "server") server(in);
+  else rounds(in);
   return 0;
 }

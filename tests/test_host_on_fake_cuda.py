@@ -27,8 +27,10 @@ def program(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     synth.pe_fastq(16 << 20, seed=12, ref_len=2_000_000).tofile(d / "in.fastq")
 
-    def run(mode):
-        r = subprocess.run([str(d / "program"), mode, str(d / "in.fastq")], capture_output=True, text=True, timeout=300)
+    synth.fasta(16 << 20, seed=12).tofile(d / "in.fasta")
+
+    def run(mode, name="in.fastq"):
+        r = subprocess.run([str(d / "program"), mode, str(d / name)], capture_output=True, text=True, timeout=300)
         assert r.returncode == 0, r.stdout + r.stderr
         return r.stdout
 
@@ -43,3 +45,11 @@ def test_calls_after_a_failure(program):
 def test_server_does_not_block_requests(program):
     """The engine's lock is free while it reads a batch's error word back."""
     assert "ok requests" in program("server")
+
+
+def test_segments_per_team_by_depth(program):
+    """Teams take two segments each in FASTQ (eight levels, many commands) and
+    one in a genome (two or three levels), where two were slower than a warp
+    per segment."""
+    assert "rounds 2" in program("rounds")
+    assert "rounds 1" in program("rounds", "in.fasta")
