@@ -733,6 +733,13 @@ constexpr uint32_t kMaxTeam = 16;  // warps per team
 constexpr uint32_t kStagedThreads = 768;
 constexpr uint32_t kStagedSmem = 228352;  // dynamic shared memory of staged_kernel; its static part is below 4 KiB
 
+// Waits for warps of the same team are not dependency waits, which L.wait_ns
+// bounds: they end by themselves, and have a limit only so that no poll is
+// endless.
+__device__ __forceinline__ uint64_t own_wait_ns(const DecodeLaunch &L) {
+  return max(L.wait_ns, (uint64_t)2000000000);
+}
+
 __device__ __forceinline__ uint32_t ld_vol(const uint32_t *p) { return *const_cast<const volatile uint32_t *>(p); }
 
 // The literals of a segment that a team's first warp is decoding, moved from
@@ -1070,7 +1077,7 @@ __device__ __forceinline__ bool match_phase_team(const DecodeLaunch &L, const De
       log2_S >= 4 && (kMode == kViewPaged  ? (reinterpret_cast<uintptr_t>(V.slot_base) & 15) == 0
                       : kMode == kViewRing ? ((reinterpret_cast<uintptr_t>(V.base) | V.origin) & 15) == 0
                                            : ((reinterpret_cast<uintptr_t>(V.base) - V.origin) & 15) == 0);
-  const uint64_t deadline = now_ns() + L.wait_ns;
+  const uint64_t begun = now_ns();
   const uint32_t B = 8 * T >= nc ? 8u : 16 * T >= nc ? 16u : 32u;
   for (uint32_t c0 = B * first; c0 < nc; c0 += B * T) {
     const uint32_t c = c0 + (uint32_t)lane;
@@ -1166,8 +1173,10 @@ __device__ __forceinline__ bool match_phase_team(const DecodeLaunch &L, const De
           continue;
         }
         uint32_t why = 0;
-        if (lane == 0 && (spin & 7) == 7)
-          why = ld_vol(&ts->fail) || ld_relaxed(L.err) ? 1u : now_ns() > deadline ? 2u : 0u;
+        if ((spin & 7) == 7) {
+          const uint64_t limit = __any_sync(kFull, pending && (f0 || f1)) ? L.wait_ns : own_wait_ns(L);
+          if (lane == 0) why = ld_vol(&ts->fail) || ld_relaxed(L.err) ? 1u : now_ns() - begun > limit ? 2u : 0u;
+        }
         why = __shfl_sync(kFull, why, 0);
         if (why) {
           if (why == 2 && lane == 0) latch(L.err, kErrTimeout);
@@ -1391,7 +1400,7 @@ __global__ void __launch_bounds__(kStagedThreads, 1) staged_kernel(DecodeLaunch 
         named_sync(team + 8, 64);
         const uint32_t s = __shfl_sync(kFull, ts->seg, 0);
         if (s < A.n_seg && !__shfl_sync(kFull, ld_vol(&ts->fail), 0) &&
-            !place_literals(st, ts, out_s, A.dir[s].n_lit, now_ns() + L.wait_ns, L.err, lane) && lane == 0)
+            !place_literals(st, ts, out_s, A.dir[s].n_lit, now_ns() + own_wait_ns(L), L.err, lane) && lane == 0)
           *const_cast<volatile uint32_t *>(&ts->fail) = 1;
       }
       team_sync();
