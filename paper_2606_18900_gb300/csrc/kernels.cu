@@ -2015,12 +2015,10 @@ __device__ __forceinline__ void copy_line_block(const RecordLines &L, uint32_t b
 #pragma unroll
   for (int v = 1; v < 4; ++v)
     if (b >= L.u[v]) line = L.to[v], from = L.from[v], len = L.ln[v], u0 = L.u[v];
-  const uint32_t al = (uint32_t)reinterpret_cast<uintptr_t>(line) & 15u, k = 16 * (b - u0);
-  // bytes [f, g) of the line fall into this block, from its byte o on
-  const uint32_t f = k ? k - al : 0u, g = min(len, k + 16 - al);
-  uint8_t *const to = line - al + k;
-  const uint32_t o = k ? 0u : al, m = g - f;
-  from += f;
+  const LineBlock part = line_block((uint32_t)reinterpret_cast<uintptr_t>(line) & 15u, len, b - u0);
+  const uint32_t o = part.o, m = part.n;
+  uint8_t *const to = line + part.from - o;
+  from += part.from;
   const uint32_t dl = (uint32_t)reinterpret_cast<uintptr_t>(from) & 15u;
   const uint4 *blk = reinterpret_cast<const uint4 *>(from - dl);
   uint4 X = make_uint4(0, 0, 0, 0), Y = X;
@@ -2070,8 +2068,7 @@ __global__ void __launch_bounds__(256) interleave_kernel(LineStreams S, uint8_t 
       for (int q = 0; q < 4; ++q) {
         L.to[q] = out + at;
         at += L.ln[q];
-        const uint32_t al = (uint32_t)reinterpret_cast<uintptr_t>(L.to[q]) & 15u;
-        L.u[q + 1] = L.u[q] + (L.ln[q] ? (al + L.ln[q] + 15) >> 4 : 0u);
+        L.u[q + 1] = L.u[q] + line_blocks((uint32_t)reinterpret_cast<uintptr_t>(L.to[q]) & 15u, L.ln[q]);
       }
       return L;
     };

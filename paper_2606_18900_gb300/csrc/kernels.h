@@ -145,6 +145,29 @@ struct GatherJob {
 // All jobs in one launch: the jobs' 64 KiB chunks are spread over the CTAs.
 cudaError_t launch_multi_gather(const GatherJob *jobs, uint32_t n_jobs, uint64_t n_chunks, cudaStream_t st);
 
+// A line copied in the output's aligned 16-byte blocks: it has len bytes (any
+// number below 2^32) and starts al bytes into a block. line_blocks: the blocks
+// that it touches; line_block: bytes [from, from + n) of it go to the b-th of
+// them, from its byte o on. Nothing here exceeds 32 bits before the true value
+// does: the sum al + len is never formed, and 16 b - al is the byte `from`
+// modulo 2^32, which is below len.
+struct LineBlock {
+  uint32_t from, n, o;
+};
+#if defined(__CUDACC__)
+#define ACE_LINE __host__ __device__ __forceinline__
+#else
+#define ACE_LINE inline
+#endif
+ACE_LINE uint32_t line_blocks(uint32_t al, uint32_t len) {
+  return len ? (len >> 4) + ((al + (len & 15u) + 15u) >> 4) : 0u;
+}
+ACE_LINE LineBlock line_block(uint32_t al, uint32_t len, uint32_t b) {
+  const uint32_t from = b ? 16u * b - al : 0u, o = b ? 0u : al, left = len - from, room = 16u - o;
+  return LineBlock{from, left < room ? left : room, o};
+}
+#undef ACE_LINE
+
 // Reassembles a FASTQ from its four decoded line streams (base[k], len[k]
 // bytes; base[k] 16-byte aligned, readable to the next multiple of 16): newline
 // index of each stream (counts: one u32 per 64 KiB chunk of every stream;

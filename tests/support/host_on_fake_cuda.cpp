@@ -11,6 +11,8 @@
 //          engine reads a batch's error word back
 //        host_on_fake_cuda rounds <file>  prints how many segments one after
 //          the other its whole-file decode allows a team
+//        host_on_fake_cuda blocks <file>  the blocks of a line (line_block),
+//          for short lines and for lines of almost 4 GiB
 // prints "ok" lines and exits 1 at the first violation.
 #include <cuda_runtime.h>
 
@@ -419,6 +421,29 @@ void server(const std::vector<uint8_t> &in) {
   std::printf("ok requests go on while an error word is read back\n");
 }
 
+// the blocks' parts follow one another, fill their blocks and end with the line
+void blocks() {
+  const auto check = [](uint32_t al, uint32_t len, uint32_t b) {
+    const LineBlock p = line_block(al, len, b);
+    const uint64_t begin = 16 * (uint64_t)b, end = begin + 16;  // of the block, al bytes before the line's start
+    const uint64_t from = std::max<uint64_t>(begin, al) - al, to = std::min<uint64_t>(end - al, len);
+    REQUIRE(p.from == from && p.n == to - from && p.o == from + al - begin && p.n >= 1 && p.o + p.n <= 16);
+  };
+  for (uint32_t al = 0; al < 16; ++al) {
+    REQUIRE(line_blocks(al, 0) == 0);
+    for (uint32_t len = 1; len < 200; ++len) {
+      REQUIRE(line_blocks(al, len) == (al + len + 15) / 16);
+      for (uint32_t b = 0; b < line_blocks(al, len); ++b) check(al, len, b);
+    }
+    for (uint32_t less = 1; less < 40; ++less) {
+      const uint32_t len = 0u - less;
+      REQUIRE(line_blocks(al, len) == ((uint64_t)al + len + 15) / 16);
+      for (uint32_t k = 0; k < 4; ++k) check(al, len, k), check(al, len, line_blocks(al, len) - 1 - k);
+    }
+  }
+  std::printf("ok blocks\n");
+}
+
 void rounds(const std::vector<uint8_t> &in) {
   const auto arc = encoded(in.data(), in.size(), 14);
   Opened o({&arc});
@@ -436,6 +461,7 @@ int main(int argc, char **argv) {
   std::vector<uint8_t> in((std::istreambuf_iterator<char>(f)), std::istreambuf_iterator<char>());
   if (std::string(argv[1]) == "calls") calls(in);
   else if (std::string(argv[1]) == "server") server(in);
+  else if (std::string(argv[1]) == "blocks") blocks();
   else rounds(in);
   return 0;
 }

@@ -53,3 +53,9 @@ def test_segments_per_team_by_depth(program):
     per segment."""
     assert "rounds 2" in program("rounds")
     assert "rounds 1" in program("rounds", "in.fasta")
+
+
+def test_blocks_of_a_line(program):
+    """The pieces in which a line is copied, up to the longest line that a
+    stream may hold: sums in 32 bits wrapped from 2^32 - 30 bytes on."""
+    assert "ok blocks" in program("blocks")
