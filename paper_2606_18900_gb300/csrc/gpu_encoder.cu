@@ -1089,11 +1089,11 @@ int gpu_encode_steps(aceapex_gpu_encoder *E, const uint8_t *in, int in_on_device
     // window have no match
     const ParseCtx g{E->in.as<uint8_t>(), n, base, S, D, log2_S, W, mm, cap, smask};
     uint64_t *table = E->mtab.as<uint64_t>();
-    ENC_TRY(cudaMemsetAsync(table, 0, 8 * (b - a), st));  // (the matches are stored, nothing else)
     match_ev.emplace_back(nullptr, nullptr);
     ENC_TRY(fresh_event(&match_ev.back().first));
     ENC_TRY(fresh_event(&match_ev.back().second));
     ENC_TRY(cudaEventRecord(match_ev.back().first, st));
+    ENC_TRY(cudaMemsetAsync(table, 0, 8 * (b - a), st));  // (the matches are stored, nothing else)
     if (lim) {
       enc_match_kernel<<<(unsigned)E->sms * 16, 256, 0, st>>>(g, K, V, lim, sentinel, a, b, table);
       ++E->launches;
