@@ -10,11 +10,13 @@
 //     hash then sit in ascending order, so the slots before a position's
 //     slot are its hash chain, latest first, equal to the chains of a
 //     sequential insertion pass over a hash table.
-//  2. match and parse: one thread per sorted slot finds the longest legal
-//     match of its position among the preceding slots (coalesced reads, no
-//     dependent walk; a candidate whose 8 bytes ending at the current best
-//     length differ cannot win and is not compared further) into a table
-//     indexed by position, with a bitmask of the usable ones; then one
+//  2. match and parse: a warp per 32 sorted slots finds the longest legal
+//     match of each one's position among the preceding slots (no dependent
+//     walk): the (slot, candidate) pairs are spread over the lanes, or, where
+//     a warp has more than 256 of them, a thread takes a slot (a candidate
+//     whose 8 bytes ending at the current best length differ cannot win there
+//     and is not compared further). The matches go into a table indexed by
+//     position, with a bitmask of the usable ones; then one
 //     thread per segment (the ruler level schedule makes segments
 //     independent) parses greedily with one-step lazy matching, jumping
 //     between mask bits, applies the symbol budget, flattens intra-segment
@@ -97,15 +99,9 @@ struct ParseCtx {
   uint32_t log2_S, W, min_match, cap, sample_mask;
 };
 
-// match_limit: how long a match of position p from candidate c may be.
-//
-// match_at_slot: longest legal match at position p = base + V[j], sorted slot j
-// (the sequential form, of which enc_match_kernel is the warp-wide one). The
-// positions with the same hash sit in the slots just before j, latest first
-// (the sort is stable), so they are p's hash chain: at most kChainDepth of
-// them are tried. A candidate is clipped at the distance bound, at the
-// segment end, at p itself (src + len <= p) and at the first source segment
-// that the level schedule forbids.
+// How long a match of position p from candidate c may be: to the segment's
+// end, to p itself (src + len <= p) and to the first source segment that the
+// level schedule forbids.
 ACE_HD uint64_t match_limit(const ParseCtx &g, uint64_t c, uint64_t p) {
   const uint64_t s = p >> g.log2_S, seg_end = min64(g.n, (s + 1) << g.log2_S);
   const uint32_t Ts = ruler_target(s, g.cap);
@@ -121,6 +117,11 @@ ACE_HD uint64_t match_limit(const ParseCtx &g, uint64_t c, uint64_t p) {
   return lim;
 }
 
+// Longest legal match at position p = base + V[j], sorted slot j (the
+// sequential form, of which enc_match_kernel is the warp-wide one). The
+// positions with the same hash sit in the slots just before j, latest first
+// (the sort is stable), so they are p's hash chain: at most kChainDepth of
+// them are tried, none beyond the distance bound, each up to match_limit.
 ACE_HD uint64_t match_at_slot(const ParseCtx &g, const uint32_t *K, const uint32_t *V, uint64_t j, uint64_t p,
                               uint64_t *src_out) {
   const uint64_t s = p >> g.log2_S, seg_end = min64(g.n, (s + 1) << g.log2_S);
@@ -450,8 +451,8 @@ __global__ void __launch_bounds__(256) rs_scatter_kernel(const uint32_t *kin, co
 // takes the first longest one of its pairs as match_at_slot would (the 8-byte
 // test there only saves comparing, so it has no counterpart here). A pair is
 // compared over kGoodEnough bytes at most: the first pair that long ends its
-// slot's walk, and only that one's full length is needed. 192 MiB of FASTQ:
-// 18.3 -> 12.9 ms.
+// slot's walk, and only that one's full length is needed. 192 MiB of FASTQ,
+// with the clearing of the table: 18.4 -> 13.1 ms.
 //
 // The length from kGoodEnough on of the match of p from c. (Out of line: few
 // slots come here; inlined it costs the kernel 0.4 ms in registers.)
@@ -461,7 +462,11 @@ __device__ __noinline__ uint64_t long_match(const ParseCtx &g, uint64_t c, uint6
 // Pairs of a warp (of at most 512) that are spread over its lanes. With more,
 // most slots have long chains: a thread per slot leaves few lanes waiting, and
 // the 8-byte test pays (16 MB of genome, min_match 32: 0.38 ms against 1.15
-// with every warp's pairs spread; 192 MiB of FASTQ 12.9 against 13.4).
+// with every warp's pairs spread; 192 MiB of FASTQ 12.9 against 13.4). Where
+// all slots have one key the pairs are not even counted, which leaves the cost
+// of this choice at 1 to 3 % in inputs made of such chains (64 MiB of one byte:
+// 7.6 ms without it, 8.0 now, 8.2 when they were counted; 500 MB of genome,
+// where these are the positions left out of sampling: 9.0, 6.7, 8.0).
 constexpr uint32_t kPairsMost = 256;
 constexpr uint32_t kMatchStop = 0xffffffffu;  // this candidate and the later ones are too far away
 constexpr uint32_t kMatchFull = 0x80000000u;  // the match reaches the end of the segment
@@ -483,24 +488,30 @@ __global__ void __launch_bounds__(256) enc_match_kernel(ParseCtx g, const uint32
     uint32_t prev = __shfl_up_sync(kFull, key, 1);
     if (lane == 0) prev = j0 ? K[j0 - 1] : ~key;
     const uint32_t equal = __ballot_sync(kFull, valid && prev == key);
-    uint32_t equal_before = 0;
-    if (equal & 1u) {  // (then j0 > 0, so j0 >= 32)
-      const uint32_t kb = K[j0 - 32 + lane];
-      uint32_t pb = __shfl_up_sync(kFull, kb, 1);
-      if (lane == 0) pb = j0 > 32 ? K[j0 - 33] : ~kb;
-      equal_before = __ballot_sync(kFull, pb == kb);
-    }
-    // candidates: the run of equal keys that ends here
-    uint32_t n = __clz((int)~(equal << (31 - lane)));
-    if (n == lane + 1) n += __clz((int)~equal_before);
-    n = active ? min(n, kChainDepth) : 0u;
-    uint32_t incl = n;
+    // n: candidates of the slot; first: its first pair; total: pairs of the
+    // warp. (32 equal keys in a row are 392 pairs or more, which need no count.)
+    uint32_t n = active, first = 0, total = kPairsMost + 1;
+    if (equal != kFull) {
+      uint32_t equal_before = 0;
+      if (equal & 1u) {  // (then j0 > 0, so j0 >= 32)
+        const uint32_t kb = K[j0 - 32 + lane];
+        uint32_t pb = __shfl_up_sync(kFull, kb, 1);
+        if (lane == 0) pb = j0 > 32 ? K[j0 - 33] : ~kb;
+        equal_before = __ballot_sync(kFull, pb == kb);
+      }
+      // candidates: the run of equal keys that ends here
+      n = __clz((int)~(equal << (31 - lane)));
+      if (n == lane + 1) n += __clz((int)~equal_before);
+      n = active ? min(n, kChainDepth) : 0u;
+      uint32_t incl = n;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(kFull, incl, o);
-      if (lane >= (uint32_t)o) incl += y;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
+      }
+      first = incl - n;
+      total = __shfl_sync(kFull, incl, 31);
     }
-    const uint32_t first = incl - n, total = __shfl_sync(kFull, incl, 31);
     if (total > kPairsMost) {
       if (n) {
         uint64_t src;
