@@ -144,6 +144,10 @@ int launch_batch_on(aceapex_server *S, Slot &slot, const std::vector<Req *> &bat
     L.epoch = slot.words.p + 1;
     L.counter = slot.words.p + 2;
     L.scratch = slot.scratch.p;
+    // (a slot without global stages: every segment fitted the shared stage when
+    // the server was made, and still does if the handle's stage was made
+    // smaller since)
+    if (!slot.scratch.p) L.stage_cap = kSmemStage;
     if ((e = launch_decode(L, A->grid, (int)kDecodeThreads, st)) != cudaSuccess) return ACEAPEX_ECUDA;
   }
   // gather every request into its caller buffer

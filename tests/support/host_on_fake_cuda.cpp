@@ -8,7 +8,8 @@
 // usage: host_on_fake_cuda calls <FASTQ file>   each entry point, with each of
 //          its runtime calls failing in turn, and then called again
 //        host_on_fake_cuda server <FASTQ file>  requests go on while the serving
-//          engine reads a batch's error word back
+//          engine reads a batch's error word back, and a handle's launch
+//          configuration may change while it is served
 //        host_on_fake_cuda rounds <file>  prints how many segments one after
 //          the other its whole-file decode allows a team
 //        host_on_fake_cuda blocks <file>  the blocks of a line (line_block),
@@ -417,6 +418,12 @@ void server(const std::vector<uint8_t> &in) {
   REQUIRE(serve(S, 50, out) == 0);
   aceapex_server_destroy(S);
   g_on_read_back = nullptr;
+  // a handle whose stage is made smaller while it is served
+  REQUIRE(aceapex_set_launch(o.as[0], 0, 0, 0) == ACEAPEX_OK);
+  REQUIRE(aceapex_server_create(o.as.data(), 1, 64 << 20, 4, &S) == ACEAPEX_OK);
+  REQUIRE(aceapex_set_launch(o.as[0], 0, 0, 16) == ACEAPEX_OK);
+  REQUIRE(serve(S, 50, out) == 0);
+  aceapex_server_destroy(S);
   take(out);
   std::printf("ok requests go on while an error word is read back\n");
 }
