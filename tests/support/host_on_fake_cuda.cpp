@@ -9,7 +9,8 @@
 //          its runtime calls failing in turn, and then called again
 //        host_on_fake_cuda server <FASTQ file>  requests go on while the serving
 //          engine reads a batch's error word back, and a handle's launch
-//          configuration may change while it is served
+//          configuration may change while it is served; batches whose end
+//          cannot be read end with an error
 //        host_on_fake_cuda rounds <file>  prints how many segments one after
 //          the other its whole-file decode allows a team
 //        host_on_fake_cuda blocks <file>  the blocks of a line (line_block),
@@ -76,6 +77,7 @@ cudaError_t take(void *p) {
   return cudaSuccess;
 }
 
+std::atomic<bool> g_lost{false}, g_unreadable{false};  // every event's, every copy to the host's error
 std::function<void()> g_on_read_back;  // called inside every copy to the host
 
 }  // namespace
@@ -97,6 +99,7 @@ cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind k) {
   if (k != cudaMemcpyDeviceToHost) REQUIRE(live(d, n));
   if (k != cudaMemcpyHostToDevice) REQUIRE(live(s, n));
   if (k == cudaMemcpyDeviceToHost && g_on_read_back) g_on_read_back();
+  if (k == cudaMemcpyDeviceToHost && g_unreadable) return cudaErrorUnknown;
   return std::memcpy(d, s, n), cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind k, cudaStream_t) {
@@ -122,7 +125,9 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t *ev, unsigned) {
 cudaError_t cudaEventDestroy(cudaEvent_t e) { return std::free(e), cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { return e ? call() : cudaErrorInvalidValue; }
 cudaError_t cudaEventSynchronize(cudaEvent_t e) { return e ? cudaSuccess : cudaErrorInvalidValue; }
-cudaError_t cudaEventQuery(cudaEvent_t e) { return e ? cudaSuccess : cudaErrorInvalidValue; }
+cudaError_t cudaEventQuery(cudaEvent_t e) {
+  return !e ? cudaErrorInvalidValue : g_lost ? cudaErrorLaunchFailure : cudaSuccess;
+}
 // (memory pools: not offered, so that buffers come from cudaMalloc)
 cudaError_t cudaMallocFromPoolAsync(void **, size_t, cudaMemPool_t, cudaStream_t) { return cudaErrorNotSupported; }
 cudaError_t cudaFreeAsync(void *, cudaStream_t) { return cudaErrorNotSupported; }
@@ -423,6 +428,13 @@ void server(const std::vector<uint8_t> &in) {
   REQUIRE(aceapex_server_create(o.as.data(), 1, 64 << 20, 4, &S) == ACEAPEX_OK);
   REQUIRE(aceapex_set_launch(o.as[0], 0, 0, 16) == ACEAPEX_OK);
   REQUIRE(serve(S, 50, out) == 0);
+  // batches whose end or whose error word cannot be read end with an error
+  for (std::atomic<bool> *f : {&g_lost, &g_unreadable}) {
+    *f = true;
+    REQUIRE(serve(S, 50, out) == 50);
+    *f = false;
+    REQUIRE(serve(S, 50, out) == 0);
+  }
   aceapex_server_destroy(S);
   take(out);
   std::printf("ok requests go on while an error word is read back\n");

@@ -30,7 +30,7 @@ def program(tmp_path_factory):
     synth.fasta(16 << 20, seed=12).tofile(d / "in.fasta")
 
     def run(mode, name="in.fastq"):
-        r = subprocess.run([str(d / "program"), mode, str(d / name)], capture_output=True, text=True, timeout=300)
+        r = subprocess.run([str(d / "program"), mode, str(d / name)], capture_output=True, text=True, timeout=120)
         assert r.returncode == 0, r.stdout + r.stderr
         return r.stdout
 
@@ -42,8 +42,11 @@ def test_calls_after_a_failure(program):
     assert out.count("ok ") == 9
 
 
-def test_server_does_not_block_requests(program):
-    """The engine's lock is free while it reads a batch's error word back."""
+def test_server(program):
+    """The engine's lock is free while it reads a batch's error word back; a
+    handle's stage may be made smaller while it is served; a batch whose event
+    or error word cannot be read ends with an error, and is waited for no
+    longer."""
     assert "ok requests" in program("server")
 
 
