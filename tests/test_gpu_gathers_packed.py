@@ -73,3 +73,18 @@ def test_lists_by_value_and_copied(log2_B):
                 a.decode_range(lo, hi, out)
                 a.check()
                 assert np.array_equal(out.cpu().numpy(), data[lo:hi])
+
+
+def test_page_table_cleared_with_the_gather_or_apart():
+    """Short ranges of 4,095 to 4,097 segments, each followed by others."""
+    import paper_2606_18900_gb300 as ace
+
+    data = np.random.default_rng(2).integers(0, 256, 20_000, dtype=np.uint8)
+    with ace.Archive(ace.encode(data, log2_B=2, min_match=8)) as a:
+        for lo, hi, segments in ((0, 16_380, 4095), (0, 16_384, 4096), (1, 16_385, 4097), (3, 5, 2), (3_000, 19_384, 4096),
+                                 (3_001, 19_385, 4097), (0, 20_000, 5000)):
+            assert a.range_closure(lo, hi)[0] == segments
+            out = torch.zeros(hi - lo, dtype=torch.uint8, device="cuda")
+            a.decode_range(lo, hi, out)
+            a.check()
+            assert np.array_equal(out.cpu().numpy(), data[lo:hi])
