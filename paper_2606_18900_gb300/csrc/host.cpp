@@ -1225,8 +1225,9 @@ int aceapex_decode_fastq_streams(aceapex_archive *const *parts, void *d_out, uin
     nat += cap[k];
   }
   // The parts decode side by side, each with its own persistent launch on a
-  // share of the SMs in proportion to its rANS symbols and commands (a command
-  // costs about as much as 85 symbols). One after the other, each ends in its
+  // share of the SMs in proportion to its cost: a literal costs 1, a command its
+  // 4 + W symbols and 80 for the match (fitted to 192 MiB of 150-base reads:
+  // 805 us with 60, 783 with 80). One after the other, each ends in its
   // own wavefront and last wave: 745 us for 192 MiB of FASTQ, against about 400
   // side by side. Part 0 runs on the caller's stream, the others on streams of
   // the handle that start after it and that it waits for. A handle that is

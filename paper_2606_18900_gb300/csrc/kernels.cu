@@ -1879,9 +1879,9 @@ __global__ void __launch_bounds__(kCrcThreads, 3) window_crc_kernel(OutView v, u
 // ------------------------------------------------- FASTQ stream separation
 // A FASTQ split into its four line streams (headers, sequences, '+' lines,
 // qualities) is put back together on the device: the newlines of each
-// decoded stream are indexed (count per chunk, scan, positions), then one warp
-// per record copies line r of every stream to its place. Record r starts at
-// the sum over the streams of the start of their line r, since every earlier
+// decoded stream are indexed (count per chunk, scan, positions), then warps take
+// eight consecutive records at a time and copy line r of every stream to its
+// place. Record r starts at the sum over the streams of the start of their line r, since every earlier
 // line of every stream precedes it in the FASTQ.
 constexpr uint32_t kNlChunk = 65536;
 
