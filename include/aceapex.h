@@ -413,7 +413,7 @@ typedef struct {
   double ms_total;    /* input copy to archive copy-out, inclusive */
   double ms_h2d;      /* input copy into the encoder's padded buffer */
   double ms_chains;   /* hashing and radix sort (all windows) */
-  double ms_match;    /* the match-search kernel (all windows) */
+  double ms_match;    /* clearing the match table and the match search (all windows) */
   double ms_parse;    /* match mask, parse, dependency lists, symbols, levels (all windows) */
   double ms_entropy;  /* tables, rANS (two passes), directory and sections */
   double ms_d2h;      /* archive copy to host memory */
