@@ -11,6 +11,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <numeric>
 #include <thread>
 #include <vector>
 
@@ -1075,8 +1076,9 @@ int aceapex_stream_range(aceapex_archive *a, uint64_t lo, uint64_t hi, uint64_t 
   std::vector<uint32_t> segs;
   for (uint64_t wa = lo; wa < hi; wa += window) {
     uint64_t wb = std::min(hi, wa + window);
-    segs.clear();
-    for (uint64_t s = wa >> h.log2_S; s <= (wb - 1) >> h.log2_S; ++s) segs.push_back((uint32_t)s);
+    const uint64_t first = wa >> h.log2_S;
+    segs.resize(((wb - 1) >> h.log2_S) + 1 - first);
+    std::iota(segs.begin(), segs.end(), (uint32_t)first);
     wstart.push_back(work.size());
     level_order(a->dir, segs.data(), segs.size(), 0, work);
   }
