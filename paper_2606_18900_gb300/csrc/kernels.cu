@@ -1802,8 +1802,9 @@ __device__ __forceinline__ uint32_t crc_raw16(const uint32_t *T, uint4 w) {
 }
 
 // CRC-32 of [lo, hi) of the ring view, written to *out by the CTA that
-// finishes last. The window is read in pieces [max(lo, seg), min(hi, seg_end)),
-// a warp per piece, persistent grid: in rows of 512 bytes, lane j taking the
+// finishes last. The window is read in the parts of it that lie in one aligned
+// piece of 2^log2_P bytes each (crc_piece says how large), a warp per piece,
+// persistent grid: in rows of 512 bytes, lane j taking the
 // 16 bytes at 512 i + 16 j of row i (coalesced), whose 16-byte pieces it folds
 // Horner-style with a shift of 512 bytes between rows; bytes after the last
 // full row are folded per lane. Each lane then shifts its register past the
@@ -1813,7 +1814,7 @@ __device__ __forceinline__ uint32_t crc_raw16(const uint32_t *T, uint4 w) {
 // joined in order (a second kernel that joined 8,192 pieces of a window in one
 // CTA took 31 us, beside 45 us of reading). sums: the register and the number
 // of CTAs done, both zero between launches.
-__global__ void __launch_bounds__(kCrcThreads, 3) window_crc_kernel(OutView v, uint32_t log2_S, uint64_t lo,
+__global__ void __launch_bounds__(kCrcThreads, 3) window_crc_kernel(OutView v, uint32_t log2_P, uint64_t lo,
                                                                     uint64_t hi, uint32_t *sums, uint32_t *out) {
   __shared__ uint32_t tab[kCrcSmemWords];
   __shared__ uint32_t s_xor;
@@ -1823,20 +1824,20 @@ __global__ void __launch_bounds__(kCrcThreads, 3) window_crc_kernel(OutView v, u
   const uint32_t *ops = tab + 4096;
   const uint32_t *op512 = ops + 1024 * 9;
   const int lane = threadIdx.x & 31;
-  const uint64_t S = uint64_t(1) << log2_S;
-  const uint64_t first = lo >> log2_S, last = (hi - 1) >> log2_S;
-  const uint64_t nseg = last - first + 1;
+  const uint64_t P = uint64_t(1) << log2_P;
+  const uint64_t first = lo >> log2_P, last = (hi - 1) >> log2_P;
+  const uint64_t pieces = last - first + 1;
   const uint32_t *all_ops = g_crc_tabs + 4096;
   uint32_t sum = 0;
-  for (uint64_t i = blockIdx.x * (uint64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < nseg;
+  for (uint64_t i = blockIdx.x * (uint64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < pieces;
        i += (uint64_t)gridDim.x * (blockDim.x >> 5)) {
     const uint64_t s = first + i;
-    const uint64_t a = (s << log2_S) > lo ? (s << log2_S) : lo;
-    const uint64_t b = ((s << log2_S) + S) < hi ? ((s << log2_S) + S) : hi;
+    const uint64_t a = (s << log2_P) > lo ? (s << log2_P) : lo;
+    const uint64_t b = ((s << log2_P) + P) < hi ? ((s << log2_P) + P) : hi;
     const uint32_t len = (uint32_t)(b - a);
     const uint8_t *p = v.base + ((a - v.origin) & v.mask);
-    // a piece with a full row has S >= 512 and starts at a multiple of S in a
-    // ring of a multiple of S bytes, so p is 16-byte aligned
+    // a piece with a full row has P >= 512; then it, and lo, start at a
+    // multiple of 16 bytes of the ring (crc_piece), so p is 16-byte aligned
     const uint32_t rows = len >> 9;
     uint32_t acc = 0;
     const uint4 *p16 = reinterpret_cast<const uint4 *>(p) + lane;
@@ -2371,18 +2372,35 @@ static cudaError_t ensure_crc_constants() {
   return e;
 }
 
+// log2 of the pieces that window_crc_kernel's warps take: 16 KiB, less where a
+// window has not that much for every warp of the grid, and never less than a
+// segment. Each piece costs a shift of its CRC past the rest of the window, up
+// to 30 dependent table steps by one lane, which is nothing beside 16 KiB and
+// more than the reading of a small segment (193 MB in 128 MiB windows, segments
+// of 64 bytes / 256 bytes / 1 KiB / 4 KiB: 3,049 / 896 / 306 / 175 us with a
+// kernel of its own to join the segments' CRCs, 3,628 / 975 / 277 / 114 with a
+// piece per segment, 98 / 97 / 98 / 97 with these). A piece lies in one part of the ring
+// (both are powers of two, from origin 0), and at 16 bytes alignment when lo does.
+static uint32_t crc_piece(const OutView &v, uint64_t lo, uint64_t bytes, uint32_t log2_S, uint64_t warps) {
+  uint32_t log2_P = log2_S;
+  if ((lo & 15) == 0 && v.origin == 0)
+    while (log2_P < 14 && (uint64_t(2) << log2_P) <= v.mask + 1 && (uint64_t(2) << log2_P) * warps <= bytes) ++log2_P;
+  return log2_P;
+}
+
 cudaError_t launch_window_crc(OutView v, uint64_t lo, uint64_t hi, uint32_t *crc, uint32_t *sums, uint32_t log2_S,
                               cudaStream_t st) {
   if (hi <= lo) return cudaSuccess;
   cudaError_t e = ensure_crc_constants();
   if (e != cudaSuccess) return e;
-  const uint64_t nseg = ((hi - 1) >> log2_S) - (lo >> log2_S) + 1;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t want = (nseg + kCrcThreads / 32 - 1) / (kCrcThreads / 32);
+  const uint32_t log2_P = crc_piece(v, lo, hi - lo, log2_S, (uint64_t)(3 * sms) * (kCrcThreads / 32));
+  const uint64_t pieces = ((hi - 1) >> log2_P) - (lo >> log2_P) + 1;
+  const uint64_t want = (pieces + kCrcThreads / 32 - 1) / (kCrcThreads / 32);
   const int grid = (int)(want < (uint64_t)(3 * sms) ? want : (uint64_t)(3 * sms));
-  window_crc_kernel<<<grid, kCrcThreads, 0, st>>>(v, log2_S, lo, hi, sums, crc);
+  window_crc_kernel<<<grid, kCrcThreads, 0, st>>>(v, log2_P, lo, hi, sums, crc);
   return cudaGetLastError();
 }
 
