@@ -351,10 +351,10 @@ DecodeLaunch base_launch(aceapex_archive *A) {
   L.stage_cap = A->stage_cap;
   L.max_stage = A->max_cmd_syms;
   // (team_shape says why) commands of a segment times levels against rANS
-  // steps of a segment, 32 symbols each: at least 1.4
+  // steps of a segment, 32 symbols each: at least 1.3, at least 0.5, or less
   const aceapex_stats &t = A->stats;
-  const uint64_t symbols = t.literal_bytes + t.n_commands * (4 + t.W);
-  L.team_rounds = 160 * t.n_commands * t.max_level >= 7 * symbols ? 2 : 1;
+  const uint64_t work = 320 * t.n_commands * t.max_level, symbols = t.literal_bytes + t.n_commands * (4 + t.W);
+  L.team_depth = work >= 13 * symbols ? 2 : work >= 5 * symbols ? 1 : 0;
   return L;
 }
 

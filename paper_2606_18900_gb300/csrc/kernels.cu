@@ -2118,12 +2118,14 @@ int decode_grid(int device, int block) {
 // beside the decode table; fewer, larger teams are faster than seven of three
 // warps (1,000 segments: 197 against 161 us).
 //
-// With more items than teams, a team decodes one segment after the other. That
-// costs a second rANS chain and saves a single warp's match phase in each level
-// of the wavefront, so it pays where the list is deep and has many commands:
-// with levels x commands per segment at least 1.4 times the rANS steps per
-// segment (L.team_rounds). us of decode_kernel -> staged_kernel, 1,824 segments
-// (two per team), by that ratio:
+// With more items than teams, teams decode a second segment after the first.
+// That costs them another rANS chain and saves a single warp's match phase in
+// each level of the wavefront, so it pays where the list is deep and has many
+// commands, which the ratio of levels x commands per segment to rANS steps per
+// segment tells: from 1.3 on (L.team_depth 2) for two segments per team, from
+// 0.5 on (1) for one segment per CTA more than teams, below for none.
+// us of decode_kernel -> staged_kernel, by that ratio:
+//   1,824 segments (12 per CTA)
 //   FASTQ, 8 levels: 16 KiB 235 -> 202 (3.1), 8 KiB 130 -> 118 (2.5), 4 KiB
 //     79 -> 76 (2.1), 2 KiB 58 -> 56 (1.9)
 //   FASTQ, 5 levels: 16 KiB 192 -> 182 (1.9), 8 KiB 107 -> 106 (1.5), 4 KiB
@@ -2131,20 +2133,27 @@ int decode_grid(int device, int block) {
 //   FASTQ, 3 levels: 16 KiB 156 -> 159 (1.1), 8 KiB 88 -> 93 (0.9)
 //   genome, 2 or 3 levels: 16 KiB 87 -> 104 (0.3), 8 KiB 53 -> 69, 4 KiB
 //     35 -> 43, 2 KiB 25 -> 35, 1 KiB 23 -> 29 (less)
+//   950 segments (7 per CTA)
+//   FASTQ, 4 levels: 16 KiB 160 -> 132 (1.3), 4 KiB 54 -> 52 (0.9)
+//   FASTQ, 3 levels: 16 KiB 143 -> 120 (1.0), 4 KiB 50 -> 47 (0.7)
+//   FASTQ, 2 levels: 16 KiB 125 -> 117 (0.6), 8 KiB 68 -> 69 (0.5), 4 KiB 44 -> 45
+//   FASTQ, 1 level: 16 KiB 103 -> 116 (0.3), 4 KiB 38 -> 44
+//   (16 KiB, 4 levels, 1,216 segments, 8 per CTA: 163 -> 154 at 1.37)
 // With one segment to a team, segments of 4 KiB and more gain or lose little (us,
 // 912 segments: FASTQ, 8 levels, 16 KiB 211 -> 163, 4 KiB 72 -> 62; 2 levels,
 // 4 KiB 43 -> 41; genome, 16 KiB 74 -> 70, 4 KiB 34 -> 37). In smaller ones the
 // chain and the match phase are short against a team's barriers and its write
-// back: 2 KiB gain in deep lists only (52 -> 48; 2 levels 30 -> 32, genome 22 ->
-// 28), 1 KiB in none (37 -> 39, 24 -> 26, 20 -> 24).
+// back: 2 KiB gain in deep lists (8 levels 52 -> 48, 304 segments 44 -> 41; 3
+// levels 34 -> 35) and lose in others (2 levels 30 -> 32, genome 22 -> 28), 1 KiB
+// lose in all (37 -> 39, 24 -> 26, 20 -> 24).
 struct Teams {
   uint32_t n, warps;
 };
 static Teams team_shape(const DecodeLaunch &L, uint32_t per_cta) {
   const uint32_t warps = std::min(L.active_warps, kStagedThreads / 32);
   const uint32_t fit = std::min((kStagedSmem - kLutBytes) / team_layout(L.arc0.log2_S, L.max_stage).bytes, kMaxTeams);
-  const bool large = L.arc0.log2_S >= 12 || (L.arc0.log2_S == 11 && L.team_rounds > 1);
-  if (!large || per_cta > L.team_rounds * fit || L.max_stage > L.stage_cap) return {0, 0};
+  const bool large = L.arc0.log2_S >= 12 || (L.arc0.log2_S == 11 && L.team_depth);
+  if (!large || per_cta > fit + (L.team_depth == 2 ? fit : L.team_depth) || L.max_stage > L.stage_cap) return {0, 0};
   const uint32_t n = std::min(per_cta, fit), T = std::min(kMaxTeam, warps / n);
   return T >= 2 ? Teams{n, T} : Teams{0, 0};
 }
@@ -2694,7 +2703,7 @@ extern "C" int aceapex_decode_all_noalloc(const void *d_archive, uint64_t nbytes
   L.active_warps = kDecodeThreads / 32;
   L.stage_cap = L.max_stage = kSmemStage;
   L.stage_need = &ctl->need;
-  L.team_rounds = 2;  // (the commands are counted on the device; FASTQ is the deep case)
+  L.team_depth = 2;  // (the commands are counted on the device; FASTQ is the deep case)
   const unsigned blocks = (unsigned)((n_seg + kNoAllocThreads - 1) / kNoAllocThreads);
   noalloc_setup_kernel<<<1, kNoAllocThreads, 0, st>>>(arc + kHeaderBytes);
   // (a reader that waits for a segment whose record is corrupt gives up: the

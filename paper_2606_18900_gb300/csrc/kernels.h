@@ -58,7 +58,7 @@ struct DecodeLaunch {
   uint32_t active_warps;    // warps per CTA that take work (<= kDecodeThreads / 32)
   uint32_t stage_cap;       // bytes of a warp's shared staging to use (<= kSmemStage)
   uint32_t max_stage;       // largest command stage (bytes) of any segment the launch may decode
-  uint32_t team_rounds;     // segments that a team of a short list may take one after the other (1 or 2)
+  uint32_t team_depth;      // how much a short list gains by teams (team_shape): 0, 1 or 2
   const uint32_t *stage_need;  // when not null: a device word with the list's largest command stage, found on the
                                // device; staged_kernel leaves the list alone when it exceeds max_stage
 };

@@ -11,8 +11,8 @@
 //          engine reads a batch's error word back, and a handle's launch
 //          configuration may change while it is served; batches whose end
 //          cannot be read end with an error
-//        host_on_fake_cuda rounds <file>  prints how many segments one after
-//          the other its whole-file decode allows a team
+//        host_on_fake_cuda depth <file>  prints the depth class of its
+//          whole-file decode (team_depth)
 //        host_on_fake_cuda blocks <file>  the blocks of a line (line_block),
 //          for short lines and for lines of almost 4 GiB
 // prints "ok" lines and exits 1 at the first violation.
@@ -140,7 +140,7 @@ cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t) { return cudaErrorNotSuppor
 namespace aceapex {
 
 int decode_grid(int, int) { return 152; }
-static uint32_t g_rounds;
+static uint32_t g_depth;
 
 static bool archive_ok(const DevArchive &A) {
   return live(A.dir, 24 * (size_t)A.n_seg) && live(A.lut, kLutBytes) && live(A.flags, 8 * (size_t)A.n_seg) &&
@@ -195,7 +195,7 @@ cudaError_t launch_decode(const DecodeLaunch &L, int grid, int, cudaStream_t) {
   if (cudaError_t r = call()) return r;
   REQUIRE(grid > 0 && archive_ok(L.arc0) && live(L.work, 8 * (size_t)L.n_work));
   REQUIRE(live(L.err, 4) && live(L.epoch, 4) && live(L.counter, 4));
-  g_rounds = L.team_rounds;
+  g_depth = L.team_depth;
   REQUIRE(L.max_stage <= L.stage_cap || live(L.scratch, (size_t)L.scratch_warps * kStageBytes));
   for (uint32_t i = 0; i < L.n_work; ++i) {
     REQUIRE(L.work[i].seg < L.arc0.n_seg);
@@ -463,13 +463,13 @@ void blocks() {
   std::printf("ok blocks\n");
 }
 
-void rounds(const std::vector<uint8_t> &in) {
+void depth(const std::vector<uint8_t> &in) {
   const auto arc = encoded(in.data(), in.size(), 14);
   Opened o({&arc});
   void *out = nullptr;
   REQUIRE(cudaMalloc(&out, in.size()) == cudaSuccess);
   REQUIRE(aceapex_decode_all(o.as[0], out, in.size(), nullptr, nullptr) == ACEAPEX_OK);
-  std::printf("rounds %u\n", g_rounds);
+  std::printf("depth %u\n", g_depth);
 }
 
 }  // namespace
@@ -481,6 +481,6 @@ int main(int argc, char **argv) {
   if (std::string(argv[1]) == "calls") calls(in);
   else if (std::string(argv[1]) == "server") server(in);
   else if (std::string(argv[1]) == "blocks") blocks();
-  else rounds(in);
+  else depth(in);
   return 0;
 }

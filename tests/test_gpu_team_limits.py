@@ -21,7 +21,7 @@ def words(n, seed):
 
 @pytest.mark.parametrize("cap", [0, 1, 8])
 @pytest.mark.parametrize("per_cta,more,log2_B", [
-    (1, 0, 12), (1, 1, 12), (6, -1, 12), (6, 0, 12), (6, 1, 12), (12, 0, 12), (12, 1, 12),
+    (1, 0, 12), (1, 1, 12), (6, -1, 12), (6, 0, 12), (6, 1, 12), (7, 0, 12), (7, 1, 12), (12, 0, 12), (12, 1, 12),
     (1, -144, 10), (6, 1, 10), (1, -144, 11), (6, 0, 11), (6, 1, 11), (12, 1, 11)])
 def test_limits(per_cta, more, log2_B, cap):
     import paper_2606_18900_gb300 as ace

@@ -50,12 +50,12 @@ def test_server(program):
     assert "ok requests" in program("server")
 
 
-def test_segments_per_team_by_depth(program):
-    """Teams take two segments each in FASTQ (eight levels, many commands) and
-    one in a genome (two or three levels), where two were slower than a warp
-    per segment."""
-    assert "rounds 2" in program("rounds")
-    assert "rounds 1" in program("rounds", "in.fasta")
+def test_depth_of_short_lists(program):
+    """Teams may take two segments each in FASTQ (eight levels, many commands)
+    and only one in a genome (two or three levels), where two were slower than
+    a warp per segment."""
+    assert "depth 2" in program("depth")
+    assert "depth 0" in program("depth", "in.fasta")
 
 
 def test_blocks_of_a_line(program):
